@@ -513,88 +513,96 @@ struct Windows {
     int32_t split;
 };
 
-// The walk over one window's quads: CTA `cta` of `ctas` takes quads
-// cta*blockDim + threadIdx, stepping by ctas*blockDim.  OBJ: where mu comes
-// from (ObjectiveSource).  OPT: the local optimiser (0 SGD, 1 Nesterov
+// The walk over one window's quads, one per thread: CTA `cta` of the window
+// takes quads cta * blockDim + threadIdx.  The grid covers every quad, so the
+// hardware hands the next CTA to whichever SM is free and the CTAs in flight
+// work on neighbouring columns; a resident grid striding over the quads let
+// them drift apart, which cost HBM locality and left a last partial round
+// (13.35 -> 12.86 ms per step on the 32-worker binary tree at d = 1.1e8, 580
+// -> 539 us on two 16-worker trees at d = 9.2M, 787 -> 683 us on the 16-worker
+// chain with regenerated centres).  OBJ: where mu
+// comes from (ObjectiveSource).  OPT: the local optimiser (0 SGD, 1 Nesterov
 // momentum, 2 Adam).  WIDE: some node has more than kRegDeg neighbours;
 // without one the wide-node paths are not compiled, and they cost the narrow
 // trees nothing.
 template <int OBJ, int OPT, bool WIDE>
 __device__ __forceinline__ void walk(const Program& prog, const ModelArgs& a, const Objective& obj,
-                                     const PhiloxKey& mu_key, int64_t cta, int64_t ctas, float4* slot_mem,
-                                     float* s_scale, float* s_fill) {
+                                     const PhiloxKey& mu_key, int64_t cta, float4* slot_mem, float* s_scale,
+                                     float* s_fill) {
     const int n = prog.n;
+    const Slots sl{slot_mem + threadIdx.x, static_cast<int>(blockDim.x)};
+    float4* cen = slot_mem + prog.nslots * blockDim.x + threadIdx.x;  // OBJ == kMuCachedCentres
+    const int64_t q = cta * blockDim.x + threadIdx.x;
+    const bool active = q < a.nquads;
+    // x (and a stored mu) of the next node in the walk are loaded one visit
+    // early, so their latency overlaps the current visit's arithmetic; the
+    // first node's, and the centres of the quad, come before the wait for the
+    // counter kernel (which writes none of them)
+    float4 xn = make_float4(0.f, 0.f, 0.f, 0.f), mn = xn;
+    if (active) {
+        xn = *reinterpret_cast<const float4*>(a.x + prog.order[0] * a.ld_x + 4 * q);
+        if (OBJ == relaysum::kMuStored) mn = ld_stream(a.mu + prog.order[0] * a.ld_x + 4 * q);
+        if (OBJ == relaysum::kMuCachedCentres)
+            for (int k = 0; k < obj.K; ++k)
+                cen[k * blockDim.x] = normal4(a.q0 + static_cast<uint32_t>(q), static_cast<uint32_t>(k), 0u, 1u, mu_key);
+    }
     wait_for_prior_grid();
     rebuild_factors(prog, a, s_scale, s_fill);
     __syncthreads();
-    const Slots sl{slot_mem + threadIdx.x, static_cast<int>(blockDim.x)};
-    float4* cen = slot_mem + prog.nslots * blockDim.x + threadIdx.x;  // OBJ == kMuCachedCentres
-    const int64_t stride = ctas * blockDim.x;
-    for (int64_t q = cta * blockDim.x + threadIdx.x; q < a.nquads; q += stride) {
-        if (OBJ == relaysum::kMuCachedCentres) {
-            for (int k = 0; k < obj.K; ++k)
-                cen[k * blockDim.x] = normal4(a.q0 + static_cast<uint32_t>(q), static_cast<uint32_t>(k), 0u,
-                                              1u, mu_key);
+    if (!active) return;
+    for (int v = 0; v < n; ++v) {
+        const int i = prog.order[v];
+        const NodeRec r = prog.node[i];
+        const float4 xv = xn;
+        const float4 mv = (OBJ == relaysum::kMuStored)
+                              ? mn : centre<OBJ>(obj, mu_key, a, i, q, cen, static_cast<int>(blockDim.x));
+        if (v + 1 < n) {  // the next node is never finalised before its own visit
+            const int inext = prog.order[v + 1];
+            xn = *reinterpret_cast<const float4*>(a.x + inext * a.ld_x + 4 * q);
+            if (OBJ == relaysum::kMuStored) mn = ld_stream(a.mu + inext * a.ld_x + 4 * q);
         }
-        // x (and a stored mu) of the next node in the walk are loaded one visit
-        // early, so their latency overlaps the current visit's arithmetic
-        float4 xn = *reinterpret_cast<const float4*>(a.x + prog.order[0] * a.ld_x + 4 * q);
-        float4 mn = (OBJ == relaysum::kMuStored) ? ld_stream(a.mu + prog.order[0] * a.ld_x + 4 * q)
-                                                  : make_float4(0.f, 0.f, 0.f, 0.f);
-        for (int v = 0; v < n; ++v) {
-            const int i = prog.order[v];
-            const NodeRec r = prog.node[i];
-            const float4 xv = xn;
-            const float4 mv = (OBJ == relaysum::kMuStored)
-                                  ? mn : centre<OBJ>(obj, mu_key, a, i, q, cen, static_cast<int>(blockDim.x));
-            if (v + 1 < n) {  // the next node is never finalised before its own visit
-                const int inext = prog.order[v + 1];
-                xn = *reinterpret_cast<const float4*>(a.x + inext * a.ld_x + 4 * q);
-                if (OBJ == relaysum::kMuStored) mn = ld_stream(a.mu + inext * a.ld_x + 4 * q);
+        // a child of a wide node p forms its incoming message as
+        // T_p - m^{t-1}_{i->p}; that row is loaded before the noise
+        // arithmetic, whose latency it then overlaps (with received sums
+        // this is the one read of m^{t-1}_{i->p})
+        float4 back = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (WIDE && (r.flags & relaysum::kRecvFromTotal)) {
+            const float* mp = a.msg_in + prog.pos_out[r.pos_base + r.parent_pos] * a.ld_m + 4 * q;
+            back = a.rsum ? ld_stream(mp) : __ldg(reinterpret_cast<const float4*>(mp));
+        }
+        const float4 z = normal4(a.q0 + static_cast<uint32_t>(q), static_cast<uint32_t>(i),
+                                 a.step, 0u, a.key);
+        const float4 xh = relayed_value<OPT>(a, i, q, xv, mv, z);
+        // the rebuild sum starts from fill_i x_i (robust rule: n - nbar_i;
+        // Alg. 6: n; Alg. 5: 1; Alg. 1: nothing)
+        float4 acc = xh;
+        if (s_fill[i] != 0.0f) acc = add4(scale4(xv, s_fill[i]), xh);
+        float4 recv = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (r.recv_slot >= 0) {
+            recv = sl[r.recv_slot];
+            if (WIDE && (r.flags & relaysum::kRecvFromTotal)) {  // m^t_{p->i} = T_p - m^{t-1}_{i->p}, written out here
+                const int e = prog.pos_in[r.pos_base + r.parent_pos];
+                recv = delivered(a, e, sub4(recv, back));
+                st_stream(a.msg_out + e * a.ld_m + 4 * q, recv);
             }
-            // a child of a wide node p forms its incoming message as
-            // T_p - m^{t-1}_{i->p}; that row is loaded before the noise
-            // arithmetic, whose latency it then overlaps (with received sums
-            // this is the one read of m^{t-1}_{i->p})
-            float4 back = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (WIDE && (r.flags & relaysum::kRecvFromTotal)) {
-                const float* mp = a.msg_in + prog.pos_out[r.pos_base + r.parent_pos] * a.ld_m + 4 * q;
-                back = a.rsum ? ld_stream(mp) : __ldg(reinterpret_cast<const float4*>(mp));
-            }
-            const float4 z = normal4(a.q0 + static_cast<uint32_t>(q), static_cast<uint32_t>(i),
-                                     a.step, 0u, a.key);
-            const float4 xh = relayed_value<OPT>(a, i, q, xv, mv, z);
-            // the rebuild sum starts from fill_i x_i (robust rule: n - nbar_i;
-            // Alg. 6: n; Alg. 5: 1; Alg. 1: nothing)
-            float4 acc = xh;
-            if (s_fill[i] != 0.0f) acc = add4(scale4(xv, s_fill[i]), xh);
-            float4 recv = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (r.recv_slot >= 0) {
-                recv = sl[r.recv_slot];
-                if (WIDE && (r.flags & relaysum::kRecvFromTotal)) {  // m^t_{p->i} = T_p - m^{t-1}_{i->p}, written out here
-                    const int e = prog.pos_in[r.pos_base + r.parent_pos];
-                    recv = delivered(a, e, sub4(recv, back));
-                    st_stream(a.msg_out + e * a.ld_m + 4 * q, recv);
-                }
-                acc = add4(acc, recv);
-            }
-            // a wide node's received sum S_i^t starts with its DFS parent's message
-            if (WIDE && a.rsum && r.deg > kRegDeg) sl[prog.rsum_slot[i]] = add4(make_float4(0.f, 0.f, 0.f, 0.f), recv);
-            switch (r.deg) {
-                case 0: break;
-                case 1: visit_small<1, WIDE>(prog, r, a, q, xh, sl, s_scale); break;
-                case 2: visit_small<2, WIDE>(prog, r, a, q, xh, sl, s_scale); break;
-                case 3: visit_small<3, WIDE>(prog, r, a, q, xh, sl, s_scale); break;
-                case 4: visit_small<4, WIDE>(prog, r, a, q, xh, sl, s_scale); break;
-                default:
-                    if (WIDE) visit_wide(prog, r, a, i, q, xh, sl, s_scale);
-                    break;
-            }
-            if (r.acc_slot < 0) {
-                st_stream(a.x + i * a.ld_x + 4 * q, scale4(acc, s_scale[i]));
-            } else {
-                sl[r.acc_slot] = acc;
-            }
+            acc = add4(acc, recv);
+        }
+        // a wide node's received sum S_i^t starts with its DFS parent's message
+        if (WIDE && a.rsum && r.deg > kRegDeg) sl[prog.rsum_slot[i]] = add4(make_float4(0.f, 0.f, 0.f, 0.f), recv);
+        switch (r.deg) {
+            case 0: break;
+            case 1: visit_small<1, WIDE>(prog, r, a, q, xh, sl, s_scale); break;
+            case 2: visit_small<2, WIDE>(prog, r, a, q, xh, sl, s_scale); break;
+            case 3: visit_small<3, WIDE>(prog, r, a, q, xh, sl, s_scale); break;
+            case 4: visit_small<4, WIDE>(prog, r, a, q, xh, sl, s_scale); break;
+            default:
+                if (WIDE) visit_wide(prog, r, a, i, q, xh, sl, s_scale);
+                break;
+        }
+        if (r.acc_slot < 0) {
+            st_stream(a.x + i * a.ld_x + 4 * q, scale4(acc, s_scale[i]));
+        } else {
+            sl[r.acc_slot] = acc;
         }
     }
 }
@@ -603,28 +611,25 @@ __device__ __forceinline__ void walk(const Program& prog, const ModelArgs& a, co
 // each copy reads its window's program and arguments at fixed parameter
 // offsets (constant operands), as the one-window kernel does; the grid's
 // first `split` CTAs take window 0.
-// Resident CTAs of 128 threads per SM the walk's registers are budgeted for
-// (0: no bound, the compiler's choice, 72 registers and 7 CTAs for the
-// stored-centre walk).  The wide-node variant runs 8 CTAs with 64 registers:
-// 6.17 -> 6.08 ms per step on the 64-worker star, while the same budget
-// slowed every narrow tree (double16 +11 %, binary32 +4 %; same-box A/B).
-template <bool WIDE>
-constexpr int kWalkMinCtas = WIDE ? 8 : 0;
-
-template <int OBJ, int OPT, int NT, bool WIDE>
-__global__ void __launch_bounds__(128, kWalkMinCtas<WIDE>)
+// MIN: the resident CTAs of 128 threads per SM that the walk's registers are
+// budgeted for (0: no bound, the compiler's choice: 64 registers, 8 CTAs).
+// The wide-node variant takes 8: 5.90 ms per step on the 64-worker star at d =
+// 2.5e7, against 6.14 ms budgeted for 7, 6.57 for 6 and 7.38 for 9 (which
+// spills).  Narrow trees with stored centres take 0 or 7 (walk_budget).
+template <int OBJ, int OPT, int NT, bool WIDE, int MIN>
+__global__ void __launch_bounds__(128, MIN)
 relay_models_kernel(const __grid_constant__ Windows<NT> win, const __grid_constant__ Objective obj,
                     const __grid_constant__ PhiloxKey mu_key) {
     extern __shared__ float4 slot_mem[];
     __shared__ float s_scale[kMaxN];
     __shared__ float s_fill[kMaxN];
     if (NT == 1) {
-        walk<OBJ, OPT, WIDE>(win.prog[0], win.a[0], obj, mu_key, blockIdx.x, gridDim.x, slot_mem, s_scale, s_fill);
+        walk<OBJ, OPT, WIDE>(win.prog[0], win.a[0], obj, mu_key, blockIdx.x, slot_mem, s_scale, s_fill);
     } else if (static_cast<int>(blockIdx.x) < win.split) {
-        walk<OBJ, OPT, WIDE>(win.prog[0], win.a[0], obj, mu_key, blockIdx.x, win.split, slot_mem, s_scale, s_fill);
+        walk<OBJ, OPT, WIDE>(win.prog[0], win.a[0], obj, mu_key, blockIdx.x, slot_mem, s_scale, s_fill);
     } else {
-        walk<OBJ, OPT, WIDE>(win.prog[NT - 1], win.a[NT - 1], obj, mu_key, blockIdx.x - win.split,
-                             gridDim.x - win.split, slot_mem, s_scale, s_fill);
+        walk<OBJ, OPT, WIDE>(win.prog[NT - 1], win.a[NT - 1], obj, mu_key, blockIdx.x - win.split, slot_mem, s_scale,
+                             s_fill);
     }
 }
 
@@ -1235,9 +1240,8 @@ int resident_ctas(int dev, int threads, size_t smem) {
 
 // The walk over NT handles' windows in one launch (NT = 1: one handle).  The
 // handles share the objective source and the local optimiser (the caller
-// checks); threads and shared memory are sized for the larger program, and
-// the CTAs are split between the windows in proportion to their quads.
-template <int OBJ, int OPT, int NT, bool WIDE>
+// checks); threads and shared memory are sized for the larger program.
+template <int OBJ, int OPT, int NT, bool WIDE, int MIN>
 int launch_models(const relay_handle* const* hs, const ModelArgs* as, cudaStream_t stream, bool after_counts) {
     int dev = 0;
     const int sms = device_sms(&dev);
@@ -1248,33 +1252,18 @@ int launch_models(const relay_handle* const* hs, const ModelArgs* as, cudaStream
     const int threads = models_threads(per_thread);
     const size_t smem = static_cast<size_t>(per_thread) * threads * 16;
     if (smem > static_cast<size_t>(kMaxSmem)) return RELAY_EUNSUPPORTED;
-    const int per_sm = resident_ctas<relay_models_kernel<OBJ, OPT, NT, WIDE>>(dev, threads, smem);
-    if (per_sm <= 0) return RELAY_ECUDA;
-    const int64_t cap = static_cast<int64_t>(sms) * per_sm;
-    int64_t want[NT], total = 0, nq = 0;
-    for (int k = 0; k < NT; ++k) {
-        want[k] = (as[k].nquads + threads - 1) / threads;
-        total += want[k];
-        nq += as[k].nquads;
-    }
+    if (resident_ctas<relay_models_kernel<OBJ, OPT, NT, WIDE, MIN>>(dev, threads, smem) <= 0) return RELAY_ECUDA;
     Windows<NT> win;
+    int64_t grid = 0;  // a quad per thread: at most 2^27 CTAs a window
     for (int k = 0; k < NT; ++k) {
+        if (k == NT - 1) win.split = static_cast<int32_t>(grid);
+        grid += (as[k].nquads + threads - 1) / threads;
         win.prog[k] = hs[k]->prog;
         win.a[k] = as[k];
     }
-    int64_t grid = total < cap ? total : cap;
-    win.split = 0;
-    if (NT == 2) {
-        int64_t split = want[0];
-        if (total > cap) {  // CTAs in proportion to the quads, at least one per window
-            split = (cap * as[0].nquads + nq / 2) / nq;
-            split = std::min(std::max<int64_t>(split, 1), cap - 1);
-        }
-        win.split = static_cast<int32_t>(split);
-    }
     const PhiloxKey mu_key =
         philox_key(static_cast<uint64_t>(hs[0]->obj.k0) | (static_cast<uint64_t>(hs[0]->obj.k1) << 32));
-    return launch_step_kernel(relay_models_kernel<OBJ, OPT, NT, WIDE>, static_cast<int>(grid), threads, smem, stream,
+    return launch_step_kernel(relay_models_kernel<OBJ, OPT, NT, WIDE, MIN>, static_cast<int>(grid), threads, smem, stream,
                               after_counts, win, hs[0]->obj, mu_key);
 }
 
@@ -1323,12 +1312,34 @@ bool has_wide(const relay_handle* h) {
     return false;
 }
 
+// Whether the walk over narrow trees with stored centres runs 7 CTAs per SM
+// rather than 8.  Eight are faster over many waves (1107 against 1125 us on
+// the 32-worker binary tree at d = 9.2M), but a short grid's last wave leaves
+// SMs idle, and it is fuller when 7 at a time divide the grid better: the
+// 64-worker torus tree at d = 1.0M is 1.61 waves of 8 or 1.84 of 7 CTAs per SM
+// and takes 283 or 272 us.
+bool seven_ctas(const ModelArgs* as, int windows) {
+    int dev = 0;
+    const int64_t sms = device_sms(&dev);
+    if (sms <= 0) return false;  // the launch reports it
+    int64_t ctas = 0;
+    for (int k = 0; k < windows; ++k) ctas += (as[k].nquads + 127) / 128;
+    auto rounds = [&](int64_t per_sm) { return (ctas + sms * per_sm - 1) / (sms * per_sm); };
+    // share of the CTA slots that the rounds fill: ctas / (rounds x slots), 7 against 8
+    return 10 * rounds(8) * 8 > 11 * rounds(7) * 7;
+}
+
 template <int OPT, int NT, bool WIDE>
 int launch_walk_src(const relay_handle* const* hs, const ModelArgs* as, cudaStream_t stream, bool after_counts) {
     switch (hs[0]->obj.source) {
-        case relaysum::kMuStored: return launch_models<relaysum::kMuStored, OPT, NT, WIDE>(hs, as, stream, after_counts);
-        case relaysum::kMuPerRow: return launch_models<relaysum::kMuPerRow, OPT, NT, WIDE>(hs, as, stream, after_counts);
-        default: return launch_models<relaysum::kMuCachedCentres, OPT, NT, WIDE>(hs, as, stream, after_counts);
+        case relaysum::kMuStored:
+            if (!WIDE && seven_ctas(as, NT))
+                return launch_models<relaysum::kMuStored, OPT, NT, WIDE, WIDE ? 8 : 7>(hs, as, stream, after_counts);
+            return launch_models<relaysum::kMuStored, OPT, NT, WIDE, WIDE ? 8 : 0>(hs, as, stream, after_counts);
+        case relaysum::kMuPerRow:
+            return launch_models<relaysum::kMuPerRow, OPT, NT, WIDE, WIDE ? 8 : 0>(hs, as, stream, after_counts);
+        default:
+            return launch_models<relaysum::kMuCachedCentres, OPT, NT, WIDE, WIDE ? 8 : 0>(hs, as, stream, after_counts);
     }
 }
 
