@@ -1,9 +1,9 @@
 """Builds librelaysum.so in-tree with nvcc for sm_103a (GB300).
 
-Three translation units compiled in parallel (host program builder, CUDA
-kernels + C ABI, host-state step), linked into one shared library with the
-CUDA runtime statically linked, so the library loads on a machine without a
-GPU.
+Translation units compiled in parallel (host program builder, C ABI with the
+setup kernels, host-state step, and the step kernels once per capacity),
+linked into one shared library with the CUDA runtime statically linked, so the
+library loads on a machine without a GPU.
 """
 from __future__ import annotations
 
@@ -19,8 +19,13 @@ INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(BUILD, "librelaysum.so")
 
-SOURCES = ["program.cpp", "relaysum.cu", "host_step.cpp"]
-HEADERS = [os.path.join(CSRC, "program.h"), os.path.join(CSRC, "handle.h"), os.path.join(INCLUDE, "relaysum.h")]
+# (source, its own flags): the step kernels are built for up to 64 workers
+# (relaysum::kSmallN) and for up to 256 (relaysum::kMaxN)
+SOURCES = [("step_kernels.cu", ["-DRELAY_CAP=256", "-DRELAY_SPACE=large"]),
+           ("step_kernels.cu", ["-DRELAY_CAP=64", "-DRELAY_SPACE=small"]),
+           ("relaysum.cu", []), ("program.cpp", []), ("host_step.cpp", [])]
+HEADERS = [os.path.join(CSRC, h) for h in ("program.h", "handle.h", "device.cuh", "step_launch.h")] + [
+    os.path.join(INCLUDE, "relaysum.h")]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-Wall",
               "-I" + INCLUDE, "-I" + CSRC]
@@ -37,7 +42,7 @@ def _stale() -> bool:
     if not os.path.exists(LIB):
         return True
     t = os.path.getmtime(LIB)
-    deps = [os.path.join(CSRC, s) for s in SOURCES] + HEADERS + [os.path.abspath(__file__)]
+    deps = [os.path.join(CSRC, s) for s, _ in SOURCES] + HEADERS + [os.path.abspath(__file__)]
     return any(os.path.getmtime(p) > t for p in deps)
 
 
@@ -49,9 +54,10 @@ def build(force: bool = False, verbose: bool = False) -> str:
     cc = nvcc()
     tag = str(os.getpid())
 
-    def compile_one(src: str) -> str:
-        obj = os.path.join(BUILD, src + f".{tag}.o")
-        cmd = [cc, *ARCH, *NVCC_FLAGS, "-c", os.path.join(CSRC, src), "-o", obj]
+    def compile_one(unit) -> str:
+        src, flags = unit
+        obj = os.path.join(BUILD, f"{src}{''.join(flags[:1])}.{tag}.o")
+        cmd = [cc, *ARCH, *NVCC_FLAGS, *flags, "-c", os.path.join(CSRC, src), "-o", obj]
         if verbose:
             cmd.insert(1, "-Xptxas=-v")
         r = subprocess.run(cmd, capture_output=True, text=True)

@@ -12,6 +12,9 @@
 struct relay_handle {
     relaysum::Program prog;
     relaysum::Objective obj;
+    // the same with room for kSmallN workers, filled when they fit
+    relaysum::SmallProgram small_prog;
+    relaysum::SmallObjective small_obj;
     int64_t d = 0, ld = 0, nquads = 0, c0 = 0;
     int64_t ld_x = 0, ld_m = 0;  // row strides (floats) of x / mu and of the messages
     int32_t mode = 1;

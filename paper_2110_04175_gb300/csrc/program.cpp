@@ -299,4 +299,38 @@ int build_program(int n, const int32_t* edges, int n_edges, Program* out, bool r
     return RELAY_OK;
 }
 
+void narrow(const Program& from, SmallProgram* to) {
+    if (from.n > kSmallN) return;
+    to->n = from.n;
+    to->E = from.E;
+    to->nslots = from.nslots;
+    to->root = from.root;
+    to->nwide = from.nwide;
+    std::copy_n(from.order, from.n, to->order);
+    std::copy_n(from.node, from.n, to->node);
+    std::copy_n(from.pos_in, from.E, to->pos_in);
+    std::copy_n(from.pos_out, from.E, to->pos_out);
+    std::copy_n(from.pos_slot, from.E, to->pos_slot);
+    std::copy_n(from.edge_src, from.E, to->edge_src);
+    std::copy_n(from.edge_dst, from.E, to->edge_dst);
+    std::copy_n(from.rb_in, from.E, to->rb_in);
+    std::copy_n(from.rsum_slot, from.n, to->rsum_slot);
+    std::copy_n(from.rsum_row, from.n, to->rsum_row);
+}
+
+void narrow(const Objective& from, SmallObjective* to) {
+    // row_off is 0 behind the workers' rows, so its largest entry is the number of non-zeros
+    const int nnz = *std::max_element(from.row_off, from.row_off + kSmallN + 1);
+    const int most = *std::max_element(from.row_off, from.row_off + kMaxN + 1);
+    if (most > nnz || nnz > kSmallMixNnz) return;
+    to->source = from.source;
+    to->K = from.K;
+    to->scale = from.scale;
+    to->k0 = from.k0;
+    to->k1 = from.k1;
+    std::copy_n(from.row_off, kSmallN + 1, to->row_off);
+    std::copy_n(from.col, nnz, to->col);
+    std::copy_n(from.w, nnz, to->w);
+}
+
 }  // namespace relaysum

@@ -66,26 +66,39 @@ struct NodeRec {        // 20 bytes; indexed by worker id
     int16_t flags;      // NodeFlags
 };
 
-struct Program {
+// N: the workers it has room for.
+template <int N>
+struct ProgramT {
+    static constexpr int kN = N, kE = 2 * (N - 1);
     int32_t n, E, nslots, root;
-    int16_t order[kMaxN];        // DFS pre-order of the workers
-    NodeRec node[kMaxN];
-    int16_t pos_in[kMaxE];       // position s of i: edge k_s -> i
-    int16_t pos_out[kMaxE];      // position s of i: edge i -> k_s
-    int16_t pos_slot[kMaxE];     // narrow node: slot of the message to child k_s; else -1
-    int16_t edge_src[kMaxE];     // directed edge e: edge_src[e] -> edge_dst[e]
-    int16_t edge_dst[kMaxE];
-    int16_t rb_in[kMaxE];        // i's positions: its incoming edges in the walk's rebuild
+    int16_t order[kN];        // DFS pre-order of the workers
+    NodeRec node[kN];
+    int16_t pos_in[kE];       // position s of i: edge k_s -> i
+    int16_t pos_out[kE];      // position s of i: edge i -> k_s
+    int16_t pos_slot[kE];     // narrow node: slot of the message to child k_s; else -1
+    int16_t edge_src[kE];     // directed edge e: edge_src[e] -> edge_dst[e]
+    int16_t edge_dst[kE];
+    int16_t rb_in[kE];        // i's positions: its incoming edges in the walk's rebuild
                                  // order (from the DFS parent, then from the children in
                                  // visit order); the node-parallel kernel adds them so
     // received sums (built only when they are on; else -1): a wide node's
     // slot of its running sum S_i^t, and its row among the sum rows (row
     // E + rsum_row[i] of a message buffer).  int8 keeps two programs within
     // one launch's parameter space.
-    int8_t rsum_slot[kMaxN];
-    int8_t rsum_row[kMaxN];
+    int8_t rsum_slot[kN];
+    int8_t rsum_row[kN];
     int32_t nwide;               // rows of received sums (0 when they are off)
 };
+
+// A handle's program has room for kMaxN workers.  Launches for up to kSmallN
+// take a copy with room for no more: kernel parameters are copied at every
+// launch and read through the constant cache.
+using Program = ProgramT<kMaxN>;
+constexpr int kSmallN = 64;
+using SmallProgram = ProgramT<kSmallN>;
+
+// Copies the program into the smaller one; a tree that does not fit is skipped.
+void narrow(const Program& from, SmallProgram* to);
 
 // Where the kernel takes the quadratic centres mu_i from.
 constexpr int kMaxMixNnz = 1024;        // non-zero mixture weights in a kernel parameter
@@ -97,15 +110,23 @@ enum ObjectiveSource : int32_t {
     kMuCachedCentres = 2,  // regenerate the K centres once per quad, then mix per row
 };
 
-struct Objective {
+template <int N, int NNZ>
+struct ObjectiveT {
     int32_t source;     // ObjectiveSource
     int32_t K;          // centres
     float scale;        // mu_i = scale * sum_k w_ik N_k
     uint32_t k0, k1;    // Philox key of the centres (stream 1)
-    int16_t row_off[kMaxN + 1];   // row i's non-zeros: [row_off[i], row_off[i+1])
-    int16_t col[kMaxMixNnz];      // centre index, ascending within a row
-    float w[kMaxMixNnz];          // weight
+    int16_t row_off[N + 1];       // row i's non-zeros: [row_off[i], row_off[i+1])
+    int16_t col[NNZ];             // centre index, ascending within a row
+    float w[NNZ];                 // weight
 };
+
+using Objective = ObjectiveT<kMaxN, kMaxMixNnz>;
+constexpr int kSmallMixNnz = 256;   // 16 workers with 10 shared centres each: 160
+using SmallObjective = ObjectiveT<kSmallN, kSmallMixNnz>;
+
+// As above: an objective with more workers or non-zeros is skipped.
+void narrow(const Objective& from, SmallObjective* to);
 
 // Status codes mirror relaysum.h.  received_sums: lay out the walk for
 // received-sum rows (one more slot per wide node).

@@ -1,0 +1,1097 @@
+// step_kernels.cu -- the kernels that run at every step: counters, the walk,
+// the node-parallel step and the multi-step kernel, and their launches.
+//
+// Compiled once per capacity (RELAY_CAP workers): the visit program and the
+// mixture of the regenerated centres ride in the kernel parameters, and their
+// arrays are sized for the capacity, so a launch for up to kSmallN workers
+// carries 3 to 7 KB instead of 13 to 32 KB.  A launch copies all of it, and
+// the tables of a small tree lie close together in the constant cache.
+//
+// Kernels:
+//   relay_counts_kernel   Alg. 1 counters, int32, one CTA, in place (lost
+//                         messages count 0; mean estimation's counts s_i).
+//   relay_models_kernel   everything per coordinate, in ONE pass over d:
+//                         local step (SGD / Nesterov / Adam) with Philox noise,
+//                         every outgoing relay message, every rebuild.  Each
+//                         x_i, mu_i and incoming message quad is read from HBM
+//                         once and each outgoing message / new model quad
+//                         written once (a child of a node of degree > 4
+//                         re-reads the one message it sent that node, see
+//                         program.h).  The path is bandwidth-bound streaming
+//                         arithmetic: no tensor cores.
+//   relay_nodes_kernel    the same step for short vectors, one thread per
+//                         (worker, quad) with the new messages exchanged in
+//                         shared memory; same bits as relay_models_kernel.
+#include "device.cuh"
+#include "step_launch.h"
+
+#include <algorithm>
+#include <cmath>
+#include <cstring>
+#include <type_traits>
+
+using relaysum::kRegDeg;
+using relaysum::NodeRec;
+
+namespace {
+
+constexpr int kMaxN = RELAY_CAP;
+constexpr int kMaxE = 2 * (kMaxN - 1);
+constexpr bool kSmall = RELAY_CAP < relaysum::kMaxN;
+using Program = relaysum::ProgramT<RELAY_CAP>;
+using Objective = std::conditional_t<kSmall, relaysum::SmallObjective, relaysum::Objective>;
+// Stored centres need none of the mixture.
+struct NoObjective {
+    int32_t K;
+};
+template <int OBJ>
+using ObjectiveArg = std::conditional_t<OBJ == relaysum::kMuStored, NoObjective, Objective>;
+
+// ------------------------------------------------- programmatic dependent launch
+
+// relay_step launches the step kernel as a programmatic dependent of the
+// counter kernel: the counter kernel lets it be scheduled at once, and the
+// step kernel waits for the counter kernel's completion (and its writes)
+// before its first read of the counters.  Launched the ordinary way, the
+// wait returns immediately.
+__device__ __forceinline__ void allow_dependent_launch() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void wait_for_prior_grid() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// ------------------------------------------------------------------ counters
+
+// c^t_{i->j} = 1 + sum_{k in N(i)\j} c^{t-1}_{k->i}: the incoming edge from
+// j is e ^ 1 for e = i -> j.  A lost message (Section 4.4) arrives as c = 0.
+// For distributed mean estimation (Alg. 5) it also adds each worker's
+// models-received count 1 + sum_j c^t_{j->i} to the running count s_i.
+// c^t of directed edge e from c^{t-1}; a lost message carries no count.
+__device__ __forceinline__ int32_t next_count(const Program& prog, const LostMask& lost, int has_lost,
+                                              const int32_t* c_old, int e) {
+    const NodeRec r = prog.node[prog.edge_src[e]];
+    int32_t s = 1;
+    for (int p = 0; p < r.deg; ++p) {
+        const int in = prog.pos_in[r.pos_base + p];
+        if (in != (e ^ 1)) s += c_old[in];
+    }
+    return (has_lost && lost(e)) ? 0 : s;
+}
+
+// The counters of NT handles (the tree windows of relay_step_windows, or one
+// handle): CTA w updates window w's.
+template <int NT>
+struct CountWindows {
+    Program prog[NT];
+    LostMask lost[NT];
+    int32_t has_lost[NT];
+    int32_t* counts[NT];
+    int64_t* dme_count[NT];  // Alg. 5's counts s_i, or null
+};
+
+template <int NT>
+__global__ void relay_counts_kernel(const __grid_constant__ CountWindows<NT> cw) {
+    allow_dependent_launch();
+    __shared__ int32_t c_old[kMaxE];
+    const int w = (NT == 1) ? 0 : static_cast<int>(blockIdx.x);
+    const Program& prog = cw.prog[w];
+    const LostMask& lost = cw.lost[w];
+    const int has_lost = cw.has_lost[w];
+    int32_t* const counts = cw.counts[w];
+    int64_t* const dme_count = cw.dme_count[w];
+    const int E = prog.E;
+    for (int e = threadIdx.x; e < E; e += blockDim.x) c_old[e] = counts[e];
+    __syncthreads();
+    for (int e = threadIdx.x; e < E; e += blockDim.x) counts[e] = next_count(prog, lost, has_lost, c_old, e);
+    if (dme_count) {  // Alg. 5: s_i += 1 + sum_j c^t_{j->i}
+        __syncthreads();
+        for (int i = threadIdx.x; i < prog.n; i += blockDim.x) {
+            const NodeRec r = prog.node[i];
+            int64_t nb = 1;
+            for (int p = 0; p < r.deg; ++p) nb += counts[prog.pos_in[r.pos_base + p]];
+            dme_count[i] += nb;
+        }
+    }
+}
+
+// The counters (and the mean-estimation counts) advanced by k steps, for
+// relay_steps: one CTA of kCountsThreads >= n threads (thread i carries
+// worker i's mean-estimation count), the counters of the two step parities
+// in shared memory, one barrier per step.
+constexpr int kCountsThreads = 256;
+static_assert(kMaxN <= kCountsThreads, "relay_counts_steps_kernel gives each worker its own thread");
+
+__global__ void __launch_bounds__(kCountsThreads)
+relay_counts_steps_kernel(const __grid_constant__ Program prog,
+                                          const __grid_constant__ LostMask lost, int has_lost, int32_t* counts,
+                                          int64_t* dme_count, int k) {
+    __shared__ int32_t c[2][kMaxE];
+    const int E = prog.E;
+    for (int e = threadIdx.x; e < E; e += blockDim.x) c[1][e] = counts[e];
+    __syncthreads();
+    int64_t received = 0;  // worker threadIdx.x: sum over the k steps of 1 + sum_j c^t_{j->i}
+    for (int j = 0; j < k; ++j) {
+        const int32_t* c_old = c[(j + 1) & 1];
+        int32_t* c_new = c[j & 1];
+        for (int e = threadIdx.x; e < E; e += blockDim.x) c_new[e] = next_count(prog, lost, has_lost, c_old, e);
+        __syncthreads();
+        if (dme_count && threadIdx.x < prog.n) {
+            const NodeRec r = prog.node[threadIdx.x];
+            int64_t nb = 1;
+            for (int p = 0; p < r.deg; ++p) nb += c_new[prog.pos_in[r.pos_base + p]];
+            received += nb;
+        }
+    }
+    for (int e = threadIdx.x; e < E; e += blockDim.x) counts[e] = c[(k - 1) & 1][e];
+    if (dme_count && threadIdx.x < prog.n) dme_count[threadIdx.x] += received;
+}
+
+// --------------------------------------------------------------- fused step
+
+// A lost message reaches its receiver as zero (Section 4.4).
+__device__ __forceinline__ float4 delivered(const ModelArgs& a, int e, float4 m) {
+    return (a.has_lost && a.lost(e)) ? make_float4(0.f, 0.f, 0.f, 0.f) : m;
+}
+
+// Per-thread view of the shared-memory slots: slot s of this thread is
+// base[s * stride]; a warp's 32 float4 of one slot are contiguous.
+struct Slots {
+    float4* base;
+    int stride;
+    __device__ __forceinline__ float4& operator[](int s) const { return base[s * stride]; }
+};
+
+// Row of wide node i's received sum in a message buffer (program.h).
+__device__ __forceinline__ int64_t rsum_row(const Program& prog, int i) { return prog.E + prog.rsum_row[i]; }
+
+// The message to the DFS parent joins the parent's accumulator (and, with
+// received sums, a wide parent's running sum S_p^t); if this worker is the
+// parent's last child, the parent's rebuild (and S_p^t) is complete.  WIDE:
+// the tree has a node of degree > kRegDeg (the walk's wide-node paths are
+// compiled only then).
+template <bool WIDE>
+__device__ __forceinline__ void to_parent(const Program& prog, const NodeRec& r, const ModelArgs& a, int64_t q,
+                                          float4 out, const Slots& sl, const float* s_scale) {
+    const float4 acc = add4(sl[r.parent_acc], out);
+    if (r.fin_parent >= 0) {
+        st_stream(a.x + r.fin_parent * a.ld_x + 4 * q, scale4(acc, s_scale[r.fin_parent]));
+    } else {
+        sl[r.parent_acc] = acc;
+    }
+    if (WIDE && a.rsum && (r.flags & relaysum::kRecvFromTotal)) {
+        const int rs = prog.rsum_slot[r.parent];
+        const float4 sum = add4(sl[rs], out);
+        if (r.fin_parent >= 0) {
+            st_stream(a.msg_out + rsum_row(prog, r.parent) * a.ld_m + 4 * q, sum);
+        } else {
+            sl[rs] = sum;
+        }
+    }
+}
+
+// Degree D <= kRegDeg: the D incoming messages live in registers; outgoing
+// message s is prefix(s) + suffix(s+1) with prefix(s) = xh + m_0 + ... + m_{s-1}.
+template <int D, bool WIDE>
+__device__ __forceinline__ void visit_small(const Program& prog, const NodeRec& r, const ModelArgs& a,
+                                            int64_t q, float4 xh, const Slots& sl,
+                                            const float* s_scale) {
+    float4 m[D];
+#pragma unroll
+    for (int s = 0; s < D; ++s) m[s] = ld_stream(a.msg_in + prog.pos_in[r.pos_base + s] * a.ld_m + 4 * q);
+    float4 pre[D];
+    pre[0] = xh;
+#pragma unroll
+    for (int s = 1; s < D; ++s) pre[s] = add4(pre[s - 1], m[s - 1]);
+    float4 suf[D];
+    suf[D - 1] = m[D - 1];
+#pragma unroll
+    for (int s = D - 2; s >= 0; --s) suf[s] = add4(m[s], suf[s + 1]);
+#pragma unroll
+    for (int s = 0; s < D; ++s) {
+        const int e = prog.pos_out[r.pos_base + s];
+        const float4 out = delivered(a, e, (s == D - 1) ? pre[s] : add4(pre[s], suf[s + 1]));
+        st_stream(a.msg_out + e * a.ld_m + 4 * q, out);
+        if (s == r.parent_pos) {
+            to_parent<WIDE>(prog, r, a, q, out, sl, s_scale);
+        } else {
+            sl[prog.pos_slot[r.pos_base + s]] = out;
+        }
+    }
+}
+
+// Degree D > kRegDeg: T = xh + the sum of all incoming messages; the message
+// to the parent is T minus the parent's incoming message, and T stays in a
+// slot for the children (see program.h).  Without received sums one
+// streaming pass reads the D incoming rows, over descending positions while
+// the children are visited in ascending order, so the first children
+// re-read the most recently read (L2-resident) rows.  With received sums,
+// T = xh + S_i^{t-1} from the one sum row, and only the parent's incoming
+// row is read here.
+__device__ __noinline__ void visit_wide(const Program& prog, const NodeRec& r, const ModelArgs& a, int i,
+                                        int64_t q, float4 xh, const Slots& sl,
+                                        const float* s_scale) {
+    const int D = r.deg;
+    const int base = r.pos_base;
+    float4 total = xh;
+    float4 from_parent = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (a.rsum) {
+        total = add4(xh, ld_stream(a.msg_in + rsum_row(prog, i) * a.ld_m + 4 * q));
+        if (r.parent_pos >= 0) from_parent = ld_stream(a.msg_in + prog.pos_in[base + r.parent_pos] * a.ld_m + 4 * q);
+    } else {
+        for (int s = D - 1; s >= 0; --s) {
+            const float4 m = ld_keep(a.msg_in + prog.pos_in[base + s] * a.ld_m + 4 * q);
+            total = add4(total, m);
+            if (s == r.parent_pos) from_parent = m;
+        }
+    }
+    if (r.parent_pos >= 0) {
+        const int e = prog.pos_out[base + r.parent_pos];
+        const float4 out = delivered(a, e, sub4(total, from_parent));
+        st_stream(a.msg_out + e * a.ld_m + 4 * q, out);
+        to_parent<true>(prog, r, a, q, out, sl, s_scale);
+    }
+    sl[r.tot_slot] = total;
+}
+
+// The local optimiser's update u (Alg. 1's local step is x^{t+1/2} = x + u):
+//   SGD:      u = -lr g
+//   Nesterov: m = beta1 m + g;  u = -lr (g + beta1 m)          (state s1 = m)
+//   Adam:     m = beta1 m + (1 - beta1) g;  v = beta2 v + (1 - beta2) g^2;
+//             u = -adam_step m / (sqrt(v) adam_ibc2 + eps)     (s1 = m, s2 = v)
+// The rule on the optimiser state (m, v) held in registers; adam_step and
+// adam_ibc2 are the factors of this step.
+template <int OPT>
+__device__ __forceinline__ float4 update_rule(const ModelArgs& a, float adam_step, float adam_ibc2, float4 g,
+                                              float4& m, float4& v) {
+    if (OPT == 0) return scale4(g, -a.lr);
+    if (OPT == 1) {
+        m = make_float4(fmaf(a.beta1, m.x, g.x), fmaf(a.beta1, m.y, g.y), fmaf(a.beta1, m.z, g.z),
+                        fmaf(a.beta1, m.w, g.w));
+        return make_float4(-a.lr * fmaf(a.beta1, m.x, g.x), -a.lr * fmaf(a.beta1, m.y, g.y),
+                           -a.lr * fmaf(a.beta1, m.z, g.z), -a.lr * fmaf(a.beta1, m.w, g.w));
+    }
+    const float c1 = 1.0f - a.beta1, c2 = 1.0f - a.beta2;
+    m = make_float4(fmaf(a.beta1, m.x, c1 * g.x), fmaf(a.beta1, m.y, c1 * g.y), fmaf(a.beta1, m.z, c1 * g.z),
+                    fmaf(a.beta1, m.w, c1 * g.w));
+    v = make_float4(fmaf(a.beta2, v.x, c2 * g.x * g.x), fmaf(a.beta2, v.y, c2 * g.y * g.y),
+                    fmaf(a.beta2, v.z, c2 * g.z * g.z), fmaf(a.beta2, v.w, c2 * g.w * g.w));
+    auto upd = [&](float mm, float vv) { return -adam_step * mm / fmaf(sqrtf(vv), adam_ibc2, a.eps); };
+    return make_float4(upd(m.x, v.x), upd(m.y, v.y), upd(m.z, v.z), upd(m.w, v.w));
+}
+
+// One step's update with the state read from and written back to HBM.
+template <int OPT>
+__device__ __forceinline__ float4 local_update(const ModelArgs& a, int i, int64_t q, float4 g) {
+    float4 m = make_float4(0.f, 0.f, 0.f, 0.f), v = m;
+    if (OPT == 0) return update_rule<OPT>(a, a.adam_step, a.adam_ibc2, g, m, v);
+    float4* pm = reinterpret_cast<float4*>(a.s1 + i * a.ld_x + 4 * q);
+    float4* pv = reinterpret_cast<float4*>(a.s2 + i * a.ld_x + 4 * q);
+    m = *pm;
+    if (OPT == 2) v = *pv;
+    const float4 u = update_rule<OPT>(a, a.adam_step, a.adam_ibc2, g, m, v);
+    __stcs(pm, m);
+    if (OPT == 2) __stcs(pv, v);
+    return u;
+}
+
+// Per-worker rebuild factors from this step's counters: x' = scale * acc
+// with acc = fill * x + x^{t+1/2} + incoming messages.
+//   mode 0: x' = acc / nbar (Alg. 1).  mode 1: x' = (acc + (n - nbar) x) / n
+//   (robust rule), the fill term folded into the accumulator up front.
+__device__ __forceinline__ void worker_factors(const ModelArgs& a, int n, int nbar, float& scale, float& fill) {
+    if (a.algo == 1) {  // x' = x + (u + sum m) / n
+        scale = 1.0f / static_cast<float>(n);
+        fill = static_cast<float>(n);
+    } else if (a.algo == 2) {  // y' = y + dhat + sum m
+        scale = 1.0f;
+        fill = 1.0f;
+    } else if (a.mode == 0) {
+        scale = 1.0f / static_cast<float>(nbar);
+        fill = 0.0f;
+    } else {
+        scale = 1.0f / static_cast<float>(n);
+        fill = static_cast<float>(n - nbar);
+    }
+}
+
+__device__ __forceinline__ void rebuild_factors(const Program& prog, const ModelArgs& a, float* s_scale,
+                                                float* s_fill) {
+    const int n = prog.n;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        const NodeRec r = prog.node[i];
+        int nbar = 1;
+        for (int p = 0; p < r.deg; ++p) nbar += __ldg(a.counts + prog.pos_in[r.pos_base + p]);
+        worker_factors(a, n, nbar, s_scale[i], s_fill[i]);
+    }
+}
+
+// The relayed value of worker i at quad q: x^{t+1/2} = x + u (Alg. 1), the
+// update u (Alg. 6) or the sample mu + sigma xi (Alg. 5), with
+// g = (x - mu) + sigma xi and z the worker's noise normals.
+// `update` maps g to u (and advances the optimiser state).
+template <typename Update>
+__device__ __forceinline__ float4 relayed_with(const ModelArgs& a, float4 xv, float4 mv, float4 z,
+                                               Update update) {
+    if (a.algo == 2)
+        return make_float4(fmaf(a.sigma, z.x, mv.x), fmaf(a.sigma, z.y, mv.y), fmaf(a.sigma, z.z, mv.z),
+                           fmaf(a.sigma, z.w, mv.w));
+    const float4 g = make_float4(fmaf(a.sigma, z.x, xv.x - mv.x), fmaf(a.sigma, z.y, xv.y - mv.y),
+                                 fmaf(a.sigma, z.z, xv.z - mv.z), fmaf(a.sigma, z.w, xv.w - mv.w));
+    const float4 u = update(g);
+    return (a.algo == 1) ? u : add4(xv, u);
+}
+
+template <int OPT>
+__device__ __forceinline__ float4 relayed_value(const ModelArgs& a, int i, int64_t q, float4 xv, float4 mv,
+                                                float4 z) {
+    return relayed_with(a, xv, mv, z, [&](float4 g) { return local_update<OPT>(a, i, q, g); });
+}
+
+// The step of NT handles in one launch: one handle, or the tree windows of
+// relay_step_windows (the double binary trees of Section 3: two trees over
+// the same workers, each carrying its own columns of the models).  The
+// grid's first `split` CTAs work on window 0, the rest on window 1.
+template <int NT>
+struct Windows {
+    Program prog[NT];
+    ModelArgs a[NT];
+    int32_t split;
+};
+
+// The walk over one window's quads, one per thread: CTA `cta` of the window
+// takes quads cta * blockDim + threadIdx.  The grid covers every quad, so the
+// hardware hands the next CTA to whichever SM is free and the CTAs in flight
+// work on neighbouring columns; a resident grid striding over the quads let
+// them drift apart, which cost HBM locality and left a last partial round
+// (13.35 -> 12.86 ms per step on the 32-worker binary tree at d = 1.1e8, 580
+// -> 539 us on two 16-worker trees at d = 9.2M, 787 -> 683 us on the 16-worker
+// chain with regenerated centres).  OBJ: where mu
+// comes from (ObjectiveSource).  OPT: the local optimiser (0 SGD, 1 Nesterov
+// momentum, 2 Adam).  WIDE: some node has more than kRegDeg neighbours;
+// without one the wide-node paths are not compiled, and they cost the narrow
+// trees nothing.
+template <int OBJ, int OPT, bool WIDE>
+__device__ __forceinline__ void walk(const Program& prog, const ModelArgs& a, const ObjectiveArg<OBJ>& obj,
+                                     const PhiloxKey& mu_key, int64_t cta, float4* slot_mem, float* s_scale,
+                                     float* s_fill) {
+    const int n = prog.n;
+    const Slots sl{slot_mem + threadIdx.x, static_cast<int>(blockDim.x)};
+    float4* cen = slot_mem + prog.nslots * blockDim.x + threadIdx.x;  // OBJ == kMuCachedCentres
+    const int64_t q = cta * blockDim.x + threadIdx.x;
+    const bool active = q < a.nquads;
+    // x (and a stored mu) of the next node in the walk are loaded one visit
+    // early, so their latency overlaps the current visit's arithmetic; the
+    // first node's, and the centres of the quad, come before the wait for the
+    // counter kernel (which writes none of them)
+    float4 xn = make_float4(0.f, 0.f, 0.f, 0.f), mn = xn;
+    if (active) {
+        xn = *reinterpret_cast<const float4*>(a.x + prog.order[0] * a.ld_x + 4 * q);
+        if (OBJ == relaysum::kMuStored) mn = ld_stream(a.mu + prog.order[0] * a.ld_x + 4 * q);
+        if (OBJ == relaysum::kMuCachedCentres)
+            for (int k = 0; k < obj.K; ++k)
+                cen[k * blockDim.x] = normal4(a.q0 + static_cast<uint32_t>(q), static_cast<uint32_t>(k), 0u, 1u, mu_key);
+    }
+    wait_for_prior_grid();
+    rebuild_factors(prog, a, s_scale, s_fill);
+    __syncthreads();
+    if (!active) return;
+    for (int v = 0; v < n; ++v) {
+        const int i = prog.order[v];
+        const NodeRec r = prog.node[i];
+        const float4 xv = xn;
+        const float4 mv = (OBJ == relaysum::kMuStored)
+                              ? mn : centre<OBJ>(obj, mu_key, a, i, q, cen, static_cast<int>(blockDim.x));
+        if (v + 1 < n) {  // the next node is never finalised before its own visit
+            const int inext = prog.order[v + 1];
+            xn = *reinterpret_cast<const float4*>(a.x + inext * a.ld_x + 4 * q);
+            if (OBJ == relaysum::kMuStored) mn = ld_stream(a.mu + inext * a.ld_x + 4 * q);
+        }
+        // a child of a wide node p forms its incoming message as
+        // T_p - m^{t-1}_{i->p}; that row is loaded before the noise
+        // arithmetic, whose latency it then overlaps (with received sums
+        // this is the one read of m^{t-1}_{i->p})
+        float4 back = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (WIDE && (r.flags & relaysum::kRecvFromTotal)) {
+            const float* mp = a.msg_in + prog.pos_out[r.pos_base + r.parent_pos] * a.ld_m + 4 * q;
+            back = a.rsum ? ld_stream(mp) : __ldg(reinterpret_cast<const float4*>(mp));
+        }
+        const float4 z = normal4(a.q0 + static_cast<uint32_t>(q), static_cast<uint32_t>(i),
+                                 a.step, 0u, a.key);
+        const float4 xh = relayed_value<OPT>(a, i, q, xv, mv, z);
+        // the rebuild sum starts from fill_i x_i (robust rule: n - nbar_i;
+        // Alg. 6: n; Alg. 5: 1; Alg. 1: nothing)
+        float4 acc = xh;
+        if (s_fill[i] != 0.0f) acc = add4(scale4(xv, s_fill[i]), xh);
+        float4 recv = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (r.recv_slot >= 0) {
+            recv = sl[r.recv_slot];
+            if (WIDE && (r.flags & relaysum::kRecvFromTotal)) {  // m^t_{p->i} = T_p - m^{t-1}_{i->p}, written out here
+                const int e = prog.pos_in[r.pos_base + r.parent_pos];
+                recv = delivered(a, e, sub4(recv, back));
+                st_stream(a.msg_out + e * a.ld_m + 4 * q, recv);
+            }
+            acc = add4(acc, recv);
+        }
+        // a wide node's received sum S_i^t starts with its DFS parent's message
+        if (WIDE && a.rsum && r.deg > kRegDeg) sl[prog.rsum_slot[i]] = add4(make_float4(0.f, 0.f, 0.f, 0.f), recv);
+        switch (r.deg) {
+            case 0: break;
+            case 1: visit_small<1, WIDE>(prog, r, a, q, xh, sl, s_scale); break;
+            case 2: visit_small<2, WIDE>(prog, r, a, q, xh, sl, s_scale); break;
+            case 3: visit_small<3, WIDE>(prog, r, a, q, xh, sl, s_scale); break;
+            case 4: visit_small<4, WIDE>(prog, r, a, q, xh, sl, s_scale); break;
+            default:
+                if (WIDE) visit_wide(prog, r, a, i, q, xh, sl, s_scale);
+                break;
+        }
+        if (r.acc_slot < 0) {
+            st_stream(a.x + i * a.ld_x + 4 * q, scale4(acc, s_scale[i]));
+        } else {
+            sl[r.acc_slot] = acc;
+        }
+    }
+}
+
+// The step kernel over NT windows.  The walk is inlined once per window, so
+// each copy reads its window's program and arguments at fixed parameter
+// offsets (constant operands), as the one-window kernel does; the grid's
+// first `split` CTAs take window 0.
+// MIN: the resident CTAs of 128 threads per SM that the walk's registers are
+// budgeted for (0: no bound, the compiler's choice: 64 registers, 8 CTAs).
+// The wide-node variant takes 8: 5.90 ms per step on the 64-worker star at d =
+// 2.5e7, against 6.14 ms budgeted for 7, 6.57 for 6 and 7.38 for 9 (which
+// spills).  Narrow trees with stored centres take 0 or 7 (walk_budget).
+template <int OBJ, int OPT, int NT, bool WIDE, int MIN>
+__global__ void __launch_bounds__(128, MIN)
+relay_models_kernel(const __grid_constant__ Windows<NT> win, const __grid_constant__ ObjectiveArg<OBJ> obj,
+                    const __grid_constant__ PhiloxKey mu_key) {
+    extern __shared__ float4 slot_mem[];
+    __shared__ float s_scale[kMaxN];
+    __shared__ float s_fill[kMaxN];
+    if (NT == 1) {
+        walk<OBJ, OPT, WIDE>(win.prog[0], win.a[0], obj, mu_key, blockIdx.x, slot_mem, s_scale, s_fill);
+    } else if (static_cast<int>(blockIdx.x) < win.split) {
+        walk<OBJ, OPT, WIDE>(win.prog[0], win.a[0], obj, mu_key, blockIdx.x, slot_mem, s_scale, s_fill);
+    } else {
+        walk<OBJ, OPT, WIDE>(win.prog[NT - 1], win.a[NT - 1], obj, mu_key, blockIdx.x - win.split, slot_mem, s_scale,
+                             s_fill);
+    }
+}
+
+// ------------------------------------------------- node-parallel fused step
+
+// For short vectors the walk leaves the GPU idle (one thread per quad walks
+// all n workers in turn), so this form of the same step gives each
+// (worker, quad) pair its own thread.  A CTA owns qb consecutive quads of
+// every worker (threads worker-major: a worker's qb quads are contiguous).
+// Phase 1: each thread forms x_i^{t+1/2} and worker i's outgoing messages
+// with the walk's arithmetic (prefix + suffix at degree <= kRegDeg, the
+// total minus the reverse message above it), writes them out and leaves
+// them in shared memory.  Phase 2, after one barrier: each thread adds its
+// worker's incoming messages in the walk's order (Program::rb_in) and
+// writes the new model.  The results equal relay_models_kernel's bit for
+// bit, and every array is still read and written once.
+
+// Degree D <= kRegDeg: outgoing message s = prefix(s) + suffix(s+1).
+template <int D>
+__device__ __forceinline__ void node_small(const Program& prog, const NodeRec& r, const ModelArgs& a,
+                                           int64_t q, float4 xh, float4* m_new, int qb) {
+    float4 m[D];
+#pragma unroll
+    for (int s = 0; s < D; ++s) m[s] = ld_stream(a.msg_in + prog.pos_in[r.pos_base + s] * a.ld_m + 4 * q);
+    float4 pre[D];
+    pre[0] = xh;
+#pragma unroll
+    for (int s = 1; s < D; ++s) pre[s] = add4(pre[s - 1], m[s - 1]);
+    float4 suf[D];
+    suf[D - 1] = m[D - 1];
+#pragma unroll
+    for (int s = D - 2; s >= 0; --s) suf[s] = add4(m[s], suf[s + 1]);
+#pragma unroll
+    for (int s = 0; s < D; ++s) {
+        const int e = prog.pos_out[r.pos_base + s];
+        const float4 out = delivered(a, e, (s == D - 1) ? pre[s] : add4(pre[s], suf[s + 1]));
+        st_stream(a.msg_out + e * a.ld_m + 4 * q, out);
+        m_new[e * qb] = out;
+    }
+}
+
+// Degree D > kRegDeg: T = x^{t+1/2} + the incoming messages summed over
+// descending positions (with received sums: + the sum row S_i^{t-1}), then
+// message s = T - (incoming message s), as in visit_wide and at the wide
+// node's children.  The incoming messages wait in shared memory (rows of
+// worker i's own incoming edges).
+__device__ __noinline__ void node_wide(const Program& prog, const NodeRec& r, const ModelArgs& a, int i,
+                                       int64_t q, float4 xh, float4* m_new, float4* m_old, int qb) {
+    const int D = r.deg;
+    const int base = r.pos_base;
+    float4 total = xh;
+    if (a.rsum) total = add4(xh, ld_stream(a.msg_in + rsum_row(prog, i) * a.ld_m + 4 * q));
+    for (int s = D - 1; s >= 0; --s) {
+        const int ein = prog.pos_in[base + s];
+        const float4 m = ld_stream(a.msg_in + ein * a.ld_m + 4 * q);
+        if (!a.rsum) total = add4(total, m);
+        m_old[ein * qb] = m;
+    }
+    for (int s = 0; s < D; ++s) {
+        const int e = prog.pos_out[base + s];
+        const float4 out = delivered(a, e, sub4(total, m_old[prog.pos_in[base + s] * qb]));
+        st_stream(a.msg_out + e * a.ld_m + 4 * q, out);
+        m_new[e * qb] = out;
+    }
+}
+
+// blockDim.x = qb * n <= 1024.  Dynamic shared memory: two [E][qb] float4
+// message buffers used by alternate blocks, plus one more for the incoming
+// messages of wide nodes when the tree has any.  With two buffers a block
+// needs one barrier: a warp already in the next block's phase 1 writes the
+// other buffer, and it can reach this buffer again only after every warp
+// has passed the next block's barrier, i.e. finished reading this one.
+template <int OBJ, int OPT>
+__global__ void __launch_bounds__(1024)
+relay_nodes_kernel(const __grid_constant__ Program prog, const __grid_constant__ ObjectiveArg<OBJ> obj,
+                   const __grid_constant__ PhiloxKey mu_key, const __grid_constant__ ModelArgs a, int qb) {
+    extern __shared__ float4 node_mem[];
+    __shared__ float s_scale[kMaxN];
+    __shared__ float s_fill[kMaxN];
+    // regenerated centres are formed per row (the walk's cached centres are
+    // the same normals mixed in the same order)
+    constexpr int kObj = (OBJ == relaysum::kMuStored) ? relaysum::kMuStored : relaysum::kMuPerRow;
+    const int i = static_cast<int>(threadIdx.x) / qb;
+    const int qi = static_cast<int>(threadIdx.x) - i * qb;
+    float4* const buf0 = node_mem + qi;                     // [e * qb]: m^t on edge e (even blocks)
+    float4* const buf1 = node_mem + prog.E * qb + qi;       // (odd blocks)
+    float4* const m_old = node_mem + 2 * prog.E * qb + qi;  // [e * qb]: m^{t-1} (wide nodes)
+    const NodeRec r = prog.node[i];
+    const float* const xrow = a.x + i * a.ld_x;
+    const float* const murow = (OBJ == relaysum::kMuStored) ? a.mu + i * a.ld_x : nullptr;
+    const int64_t nblk = (a.nquads + qb - 1) / qb;
+    const int64_t qstep = static_cast<int64_t>(gridDim.x) * qb;
+    // x (and a stored mu) of this thread's next block are loaded one block
+    // early, so their latency overlaps the barrier and the rebuild
+    float4 xn = make_float4(0.f, 0.f, 0.f, 0.f), mn = xn;
+    int64_t q = static_cast<int64_t>(blockIdx.x) * qb + qi;
+    if (q < a.nquads) {
+        xn = *reinterpret_cast<const float4*>(xrow + 4 * q);
+        if (OBJ == relaysum::kMuStored) mn = ld_stream(murow + 4 * q);
+    }
+    // Phase 1 needs no counter: the first block's runs before the wait for the
+    // counter kernel (programmatic dependent launch), overlapping it; only the
+    // rebuild factors of phase 2 need the counters, which the counter kernel
+    // writes (it writes nothing phase 1 reads).
+    bool counted = false;
+    int parity = 0;
+    for (int64_t b = blockIdx.x; b < nblk; b += gridDim.x, q += qstep, parity ^= 1) {
+        float4* const m_new = parity ? buf1 : buf0;
+        const bool active = q < a.nquads;
+        const float4 xv = xn, ms = mn;
+        if (q + qstep < a.nquads) {
+            xn = *reinterpret_cast<const float4*>(xrow + 4 * (q + qstep));
+            if (OBJ == relaysum::kMuStored) mn = ld_stream(murow + 4 * (q + qstep));
+        }
+        float4 xh = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (active) {
+            const float4 mv = (OBJ == relaysum::kMuStored) ? ms : centre<kObj>(obj, mu_key, a, i, q, nullptr, 0);
+            const float4 z = normal4(a.q0 + static_cast<uint32_t>(q), static_cast<uint32_t>(i), a.step, 0u,
+                                     a.key);
+            xh = relayed_value<OPT>(a, i, q, xv, mv, z);
+            switch (r.deg) {
+                case 0: break;
+                case 1: node_small<1>(prog, r, a, q, xh, m_new, qb); break;
+                case 2: node_small<2>(prog, r, a, q, xh, m_new, qb); break;
+                case 3: node_small<3>(prog, r, a, q, xh, m_new, qb); break;
+                case 4: node_small<4>(prog, r, a, q, xh, m_new, qb); break;
+                default: node_wide(prog, r, a, i, q, xh, m_new, m_old, qb); break;
+            }
+        }
+        if (!counted) {
+            wait_for_prior_grid();
+            rebuild_factors(prog, a, s_scale, s_fill);
+            counted = true;
+        }
+        __syncthreads();  // also publishes the factors
+        if (active) {
+            // the rebuild sum starts from fill_i x_i + x^{t+1/2}, as in the walk
+            float4 acc = xh;
+            if (s_fill[i] != 0.0f) acc = add4(scale4(xv, s_fill[i]), xh);
+            if (a.rsum && r.deg > kRegDeg) {  // and the wide node's received sum S_i^t, in the same order
+                float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
+                for (int k = 0; k < r.deg; ++k) {
+                    const float4 m = m_new[prog.rb_in[r.pos_base + k] * qb];
+                    acc = add4(acc, m);
+                    sum = add4(sum, m);
+                }
+                st_stream(a.msg_out + rsum_row(prog, i) * a.ld_m + 4 * q, sum);
+            } else {
+                for (int k = 0; k < r.deg; ++k) acc = add4(acc, m_new[prog.rb_in[r.pos_base + k] * qb]);
+            }
+            st_stream(a.x + i * a.ld_x + 4 * q, scale4(acc, s_scale[i]));
+        }
+    }
+}
+
+// ------------------------------------------------ several steps per launch
+
+// relay_steps: k consecutive steps in one launch, in the node-parallel
+// layout.  Every coordinate evolves on its own (the counters are the same
+// for all of them), so a CTA carries its qb quads of every worker through
+// all k steps without hearing from another CTA: models, centres and
+// optimiser state stay in registers, the messages of the step just taken
+// in shared memory, and the CTA advances its own copy of the counters.  HBM
+// is read once (x, mu, the optimiser state, m^{t0-1}) and written once (x,
+// the state, and the messages of the last two steps, which k relay_step
+// calls leave in the two buffers).  Each step is the node kernel's
+// arithmetic in the node kernel's order, so the result equals k relay_step
+// calls bit for bit.
+// Outgoing messages of worker i from its incoming ones in shared memory
+// (`prev`, this thread's column), with node_small's / node_wide's arithmetic.
+// They go to `cur`, and to HBM at `out` (row e at out + e * ld_m) unless null.
+template <int D>
+__device__ __forceinline__ void fused_small(const Program& prog, const NodeRec& r, const ModelArgs& a, float4 xh,
+                                            const float4* prev, float4* cur, int qb, float* out,
+                                            uint32_t lost_bits) {
+    float4 m[D];
+#pragma unroll
+    for (int s = 0; s < D; ++s) m[s] = prev[prog.pos_in[r.pos_base + s] * qb];
+    float4 pre[D];
+    pre[0] = xh;
+#pragma unroll
+    for (int s = 1; s < D; ++s) pre[s] = add4(pre[s - 1], m[s - 1]);
+    float4 suf[D];
+    suf[D - 1] = m[D - 1];
+#pragma unroll
+    for (int s = D - 2; s >= 0; --s) suf[s] = add4(m[s], suf[s + 1]);
+#pragma unroll
+    for (int s = 0; s < D; ++s) {
+        const int e = prog.pos_out[r.pos_base + s];
+        const float4 o = ((lost_bits >> s) & 1u) ? make_float4(0.f, 0.f, 0.f, 0.f)
+                                                 : ((s == D - 1) ? pre[s] : add4(pre[s], suf[s + 1]));
+        cur[e * qb] = o;
+        if (out) st_stream(out + e * a.ld_m, o);
+    }
+}
+
+// The rebuild sum: acc plus the incoming messages of step j in rb_in order.
+template <int D>
+__device__ __forceinline__ float4 fused_rebuild(const Program& prog, const NodeRec& r, const float4* cur, int qb,
+                                                float4 acc) {
+#pragma unroll
+    for (int k = 0; k < D; ++k) acc = add4(acc, cur[prog.rb_in[r.pos_base + k] * qb]);
+    return acc;
+}
+
+__device__ __noinline__ void fused_wide(const Program& prog, const NodeRec& r, const ModelArgs& a, float4 xh,
+                                        const float4* prev, float4* cur, int qb, float* out) {
+    const int D = r.deg;
+    const int base = r.pos_base;
+    float4 total = xh;
+    for (int s = D - 1; s >= 0; --s) total = add4(total, prev[prog.pos_in[base + s] * qb]);
+    for (int s = 0; s < D; ++s) {
+        const int e = prog.pos_out[base + s];
+        const float4 o = delivered(a, e, sub4(total, prev[prog.pos_in[base + s] * qb]));
+        cur[e * qb] = o;
+        if (out) st_stream(out + e * a.ld_m, o);
+    }
+}
+
+// blockDim.x = qb * n <= 1024, threads worker-major as in relay_nodes_kernel.
+// Dynamic shared memory: two [E][qb] float4 message buffers, buffer j & 1
+// holding the messages of step t0 + j (buffer 1 starts with m^{t0-1}), then
+// the rebuild factors (scale, fill) of every worker and step, [k][n] float2.
+// The counters, hence the factors, are the same for every quad: the CTA
+// advances them through the k steps once, before its first quads.  One
+// barrier per step: a thread can write a buffer again only two steps later,
+// after every thread has passed the barrier between, i.e. finished reading it.
+template <int OBJ, int OPT>
+__global__ void __launch_bounds__(1024)
+relay_fused_steps_kernel(const __grid_constant__ Program prog, const __grid_constant__ ObjectiveArg<OBJ> obj,
+                         const __grid_constant__ PhiloxKey mu_key, const __grid_constant__ ModelArgs a,
+                         const __grid_constant__ FusedSteps fs, int qb) {
+    extern __shared__ float4 fused_mem[];
+    __shared__ int32_t c_mem[2][kMaxE];  // counters of the step parities
+    constexpr int kObj = (OBJ == relaysum::kMuStored) ? relaysum::kMuStored : relaysum::kMuPerRow;
+    const int tid = static_cast<int>(threadIdx.x);
+    const int i = tid / qb;
+    const int qi = tid - i * qb;
+    const int n = prog.n;
+    const int E = prog.E;
+    const NodeRec r = prog.node[i];
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    float2* const factors = reinterpret_cast<float2*>(fused_mem + 2 * E * qb);  // [j * n + i]
+    // bit s: the message to this worker's neighbour s is lost (narrow nodes)
+    uint32_t lost_bits = 0;
+    if (a.has_lost && r.deg <= kRegDeg)
+        for (int s = 0; s < r.deg; ++s) lost_bits |= (a.lost(prog.pos_out[r.pos_base + s]) ? 1u : 0u) << s;
+    for (int e = tid; e < E; e += blockDim.x) c_mem[1][e] = a.counts[e];  // c^{t0-1}
+    __syncthreads();
+    for (int j = 0; j < fs.k; ++j) {
+        const int32_t* const c_old = c_mem[(j + 1) & 1];
+        int32_t* const c_new = c_mem[j & 1];
+        for (int e = tid; e < E; e += blockDim.x) c_new[e] = next_count(prog, a.lost, a.has_lost, c_old, e);
+        __syncthreads();
+        for (int w = tid; w < n; w += blockDim.x) {
+            const NodeRec rw = prog.node[w];
+            int nbar = 1;
+            for (int p = 0; p < rw.deg; ++p) nbar += c_new[prog.pos_in[rw.pos_base + p]];
+            float scale, fill;
+            worker_factors(a, n, nbar, scale, fill);
+            factors[j * n + w] = make_float2(scale, fill);
+        }
+    }
+    const int64_t nblk = (a.nquads + qb - 1) / qb;
+    for (int64_t b = blockIdx.x; b < nblk; b += gridDim.x) {
+        const int64_t q = b * qb + qi;
+        const bool active = q < a.nquads;
+        // m^{t0-1} of this CTA's quads (coalesced rows of qb quads) into buffer 1
+        for (int idx = tid; idx < E * qb; idx += blockDim.x) {
+            const int e = idx / qb;
+            const int64_t qg = b * qb + (idx - e * qb);
+            fused_mem[E * qb + idx] = qg < a.nquads ? ld_stream(a.msg_in + e * a.ld_m + 4 * qg) : zero;
+        }
+        float4 xv = zero, mv = zero, m1 = zero, m2 = zero;
+        if (active) {
+            xv = *reinterpret_cast<const float4*>(a.x + i * a.ld_x + 4 * q);
+            mv = (OBJ == relaysum::kMuStored) ? ld_stream(a.mu + i * a.ld_x + 4 * q)
+                                               : centre<kObj>(obj, mu_key, a, i, q, nullptr, 0);
+            if (OPT >= 1) m1 = *reinterpret_cast<const float4*>(a.s1 + i * a.ld_x + 4 * q);
+            if (OPT == 2) m2 = *reinterpret_cast<const float4*>(a.s2 + i * a.ld_x + 4 * q);
+        }
+        __syncthreads();
+        for (int j = 0; j < fs.k; ++j) {
+            float4* const cur = fused_mem + (j & 1) * E * qb + qi;
+            const float4* const prev = fused_mem + ((j + 1) & 1) * E * qb + qi;
+            float4 xh = zero;
+            if (active) {
+                const float4 z = normal4(a.q0 + static_cast<uint32_t>(q), static_cast<uint32_t>(i),
+                                         a.step + static_cast<uint32_t>(j), 0u, a.key);
+                const float st = fs.adam_step[j], ib = fs.adam_ibc2[j];
+                xh = relayed_with(a, xv, mv, z, [&](float4 g) { return update_rule<OPT>(a, st, ib, g, m1, m2); });
+                float* const out = (E > 0 && j + 2 >= fs.k) ? fs.msg[(j + 1) & 1] + 4 * q : nullptr;
+                switch (r.deg) {
+                    case 0: break;
+                    case 1: fused_small<1>(prog, r, a, xh, prev, cur, qb, out, lost_bits); break;
+                    case 2: fused_small<2>(prog, r, a, xh, prev, cur, qb, out, lost_bits); break;
+                    case 3: fused_small<3>(prog, r, a, xh, prev, cur, qb, out, lost_bits); break;
+                    case 4: fused_small<4>(prog, r, a, xh, prev, cur, qb, out, lost_bits); break;
+                    default: fused_wide(prog, r, a, xh, prev, cur, qb, out); break;
+                }
+            }
+            __syncthreads();
+            if (active) {
+                const float2 f = factors[j * n + i];  // (scale, fill)
+                float4 acc = xh;
+                if (f.y != 0.0f) acc = add4(scale4(xv, f.y), xh);
+                switch (r.deg) {
+                    case 0: break;
+                    case 1: acc = fused_rebuild<1>(prog, r, cur, qb, acc); break;
+                    case 2: acc = fused_rebuild<2>(prog, r, cur, qb, acc); break;
+                    case 3: acc = fused_rebuild<3>(prog, r, cur, qb, acc); break;
+                    case 4: acc = fused_rebuild<4>(prog, r, cur, qb, acc); break;
+                    default:
+                        for (int k = 0; k < r.deg; ++k) acc = add4(acc, cur[prog.rb_in[r.pos_base + k] * qb]);
+                        break;
+                }
+                xv = scale4(acc, f.x);
+            }
+        }
+        if (active) {
+            st_stream(a.x + i * a.ld_x + 4 * q, xv);
+            if (OPT >= 1) st_stream(a.s1 + i * a.ld_x + 4 * q, m1);
+            if (OPT == 2) st_stream(a.s2 + i * a.ld_x + 4 * q, m2);
+        }
+        __syncthreads();  // the next block refills buffer 1
+    }
+}
+
+// ------------------------------------------------------------------ launches
+
+[[maybe_unused]] const relaysum::Program& pick(const relay_handle* h, const relaysum::Program*) { return h->prog; }
+[[maybe_unused]] const relaysum::SmallProgram& pick(const relay_handle* h, const relaysum::SmallProgram*) { return h->small_prog; }
+[[maybe_unused]] const relaysum::Objective& pick(const relay_handle* h, const relaysum::Objective*) { return h->obj; }
+[[maybe_unused]] const relaysum::SmallObjective& pick(const relay_handle* h, const relaysum::SmallObjective*) { return h->small_obj; }
+[[maybe_unused]] NoObjective pick(const relay_handle*, const NoObjective*) { return NoObjective{0}; }
+
+// The handle's program and objective at this capacity.
+const Program& program_of(const relay_handle* h) { return pick(h, static_cast<const Program*>(nullptr)); }
+template <int OBJ>
+ObjectiveArg<OBJ> objective_of(const relay_handle* h) {
+    return pick(h, static_cast<const ObjectiveArg<OBJ>*>(nullptr));
+}
+
+// Launches a step kernel; `after_counts` makes it a programmatic dependent of
+// the counter kernel just enqueued on the same stream (relay_step only).
+template <typename... Params, typename... Args>
+int launch_step_kernel(void (*kernel)(Params...), int grid, int threads, size_t smem, cudaStream_t stream,
+                       bool after_counts, Args... args) {
+    if (!after_counts) {
+        kernel<<<grid, threads, smem, stream>>>(args...);
+        return launch_status();
+    }
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(static_cast<unsigned>(grid));
+    cfg.blockDim = dim3(static_cast<unsigned>(threads));
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (cudaLaunchKernelEx(&cfg, kernel, args...) != cudaSuccess) return RELAY_ECUDA;
+    return launch_status();
+}
+
+// Whether a tree has a node of degree > kRegDeg (the walk's WIDE variant).
+bool has_wide(const relay_handle* h) {
+    for (int i = 0; i < h->prog.n; ++i)
+        if (h->prog.node[i].deg > kRegDeg) return true;
+    return false;
+}
+
+// Threads per CTA for the fused kernel: 128, fewer when the slots would not
+// fit in shared memory.
+int models_threads(int nslots) {
+    int t = 128;
+    while (t > 32 && static_cast<int64_t>(nslots) * t * 16 > kMaxSmem) t -= 32;
+    return t;
+}
+
+// Opts `Kernel` in to the dynamic shared memory it may use (kMaxSmem, less
+// when its static shared memory and kMaxSmem would pass the device's per-CTA
+// limit) once per device, and returns its resident CTAs per SM for
+// (threads, smem).  Both are cached per device (queried once, not per step:
+// steps may be captured into CUDA graphs); each kernel instantiation has its
+// own cache.  0 on a CUDA error, which is cleared so that it is not reported
+// again by a later launch.
+template <auto Kernel>
+int resident_ctas(int dev, int threads, size_t smem) {
+    static std::atomic<bool> smem_set[kMaxDevices];
+    if (dev >= kMaxDevices || !smem_set[dev].load()) {
+        cudaFuncAttributes fa;
+        int optin = 0;
+        if (cudaFuncGetAttributes(&fa, Kernel) != cudaSuccess ||
+            cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) {
+            (void)cudaGetLastError();
+            return 0;
+        }
+        const int room = optin - static_cast<int>(fa.sharedSizeBytes);
+        if (room <= 0 ||
+            cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 room < kMaxSmem ? room : kMaxSmem) != cudaSuccess) {
+            (void)cudaGetLastError();
+            return 0;
+        }
+        if (dev < kMaxDevices) smem_set[dev].store(true);
+    }
+    static std::atomic<int64_t> occ_cache[kMaxDevices];
+    const int64_t key = static_cast<int64_t>(smem) * 1024 + threads;
+    const int64_t cached = dev < kMaxDevices ? occ_cache[dev].load() : 0;
+    if (cached != 0 && (cached >> 8) == key) return static_cast<int>(cached & 0xFF);
+    int per_sm = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, Kernel, threads, smem) != cudaSuccess || per_sm <= 0) {
+        (void)cudaGetLastError();
+        return 0;
+    }
+    if (dev < kMaxDevices) occ_cache[dev].store((key << 8) | (per_sm & 0xFF));
+    return per_sm;
+}
+
+// The walk over NT handles' windows in one launch (NT = 1: one handle).  The
+// handles share the objective source and the local optimiser (the caller
+// checks); threads and shared memory are sized for the larger program.
+template <int OBJ, int OPT, int NT, bool WIDE, int MIN>
+int launch_models(const relay_handle* const* hs, const ModelArgs* as, cudaStream_t stream, bool after_counts) {
+    int dev = 0;
+    const int sms = device_sms(&dev);
+    if (sms <= 0) return RELAY_ECUDA;
+    int per_thread = 0;
+    for (int k = 0; k < NT; ++k)
+        per_thread = std::max(per_thread, hs[k]->prog.nslots + (OBJ == relaysum::kMuCachedCentres ? hs[k]->obj.K : 0));
+    const int threads = models_threads(per_thread);
+    const size_t smem = static_cast<size_t>(per_thread) * threads * 16;
+    if (smem > static_cast<size_t>(kMaxSmem)) return RELAY_EUNSUPPORTED;
+    if (resident_ctas<relay_models_kernel<OBJ, OPT, NT, WIDE, MIN>>(dev, threads, smem) <= 0) return RELAY_ECUDA;
+    Windows<NT> win;
+    int64_t grid = 0;  // a quad per thread: at most 2^27 CTAs a window
+    for (int k = 0; k < NT; ++k) {
+        if (k == NT - 1) win.split = static_cast<int32_t>(grid);
+        grid += (as[k].nquads + threads - 1) / threads;
+        win.prog[k] = program_of(hs[k]);
+        win.a[k] = as[k];
+    }
+    const PhiloxKey mu_key =
+        philox_key(static_cast<uint64_t>(hs[0]->obj.k0) | (static_cast<uint64_t>(hs[0]->obj.k1) << 32));
+    return launch_step_kernel(relay_models_kernel<OBJ, OPT, NT, WIDE, MIN>, static_cast<int>(grid), threads, smem, stream,
+                              after_counts, win, objective_of<OBJ>(hs[0]), mu_key);
+}
+
+// Quads per CTA of the node-parallel kernel, threads = qb * n <= 1024: a
+// whole warp per worker up to n = 16 (every per-worker table read is then
+// warp-uniform), half a warp up to 64, then 8 and 4 quads.
+int nodes_qb(int n) { return n <= 16 ? 32 : n <= 64 ? 16 : n <= 128 ? 8 : 4; }
+
+template <int OBJ, int OPT>
+int launch_nodes(const relay_handle* h, const ModelArgs& a, cudaStream_t stream, bool after_counts) {
+    int dev = 0;
+    const int sms = device_sms(&dev);
+    if (sms <= 0) return RELAY_ECUDA;
+    const int qb = nodes_qb(h->prog.n);
+    const int threads = qb * h->prog.n;
+    bool wide = false;
+    for (int i = 0; i < h->prog.n; ++i) wide = wide || h->prog.node[i].deg > kRegDeg;
+    const size_t smem = static_cast<size_t>(wide ? 3 : 2) * h->prog.E * qb * 16;
+    if (smem > static_cast<size_t>(kMaxSmem)) return RELAY_EUNSUPPORTED;
+    const int per_sm = resident_ctas<relay_nodes_kernel<OBJ, OPT>>(dev, threads, smem);
+    if (per_sm <= 0) return RELAY_ECUDA;
+    const int64_t want = (a.nquads + qb - 1) / qb;
+    const int64_t cap = static_cast<int64_t>(sms) * per_sm;
+    const int grid = static_cast<int>(want < cap ? want : cap);
+    const PhiloxKey mu_key = philox_key(static_cast<uint64_t>(h->obj.k0) | (static_cast<uint64_t>(h->obj.k1) << 32));
+    return launch_step_kernel(relay_nodes_kernel<OBJ, OPT>, grid, threads, smem, stream, after_counts,
+                              program_of(h), objective_of<OBJ>(h), mu_key, a, qb);
+}
+
+// Whether the walk over narrow trees with stored centres runs 7 CTAs per SM
+// rather than 8.  Eight are faster over many waves (1107 against 1125 us on
+// the 32-worker binary tree at d = 9.2M), but a short grid's last wave leaves
+// SMs idle, and it is fuller when 7 at a time divide the grid better: the
+// 64-worker torus tree at d = 1.0M is 1.61 waves of 8 or 1.84 of 7 CTAs per SM
+// and takes 283 or 272 us.
+bool seven_ctas(const ModelArgs* as, int windows) {
+    int dev = 0;
+    const int64_t sms = device_sms(&dev);
+    if (sms <= 0) return false;  // the launch reports it
+    int64_t ctas = 0;
+    for (int k = 0; k < windows; ++k) ctas += (as[k].nquads + 127) / 128;
+    auto rounds = [&](int64_t per_sm) { return (ctas + sms * per_sm - 1) / (sms * per_sm); };
+    // share of the CTA slots that the rounds fill: ctas / (rounds x slots), 7 against 8
+    return 10 * rounds(8) * 8 > 11 * rounds(7) * 7;
+}
+
+template <int OPT, int NT, bool WIDE>
+int launch_walk_src(const relay_handle* const* hs, const ModelArgs* as, cudaStream_t stream, bool after_counts) {
+    switch (hs[0]->obj.source) {
+        case relaysum::kMuStored:
+            if (!WIDE && seven_ctas(as, NT))
+                return launch_models<relaysum::kMuStored, OPT, NT, WIDE, WIDE ? 8 : 7>(hs, as, stream, after_counts);
+            return launch_models<relaysum::kMuStored, OPT, NT, WIDE, WIDE ? 8 : 0>(hs, as, stream, after_counts);
+        case relaysum::kMuPerRow:
+            return launch_models<relaysum::kMuPerRow, OPT, NT, WIDE, WIDE ? 8 : 0>(hs, as, stream, after_counts);
+        default:
+            return launch_models<relaysum::kMuCachedCentres, OPT, NT, WIDE, WIDE ? 8 : 0>(hs, as, stream, after_counts);
+    }
+}
+
+// One handle: the WIDE variant when its tree has a wide node.  Several
+// windows (relay_step_windows) launch together only when none has one.
+template <int OPT, int NT>
+int launch_walk_obj(const relay_handle* const* hs, const ModelArgs* as, cudaStream_t stream, bool after_counts) {
+    if (NT == 1 && has_wide(hs[0])) return launch_walk_src<OPT, 1, true>(hs, as, stream, after_counts);
+    return launch_walk_src<OPT, NT, false>(hs, as, stream, after_counts);
+}
+
+template <int OPT>
+int launch_models_obj(const relay_handle* h, const ModelArgs& a, bool nodes, cudaStream_t stream, bool after_counts) {
+    if (nodes) {
+        if (h->obj.source == relaysum::kMuStored)
+            return launch_nodes<relaysum::kMuStored, OPT>(h, a, stream, after_counts);
+        return launch_nodes<relaysum::kMuPerRow, OPT>(h, a, stream, after_counts);
+    }
+    return launch_walk_obj<OPT, 1>(&h, &a, stream, after_counts);
+}
+
+// Quads per CTA of relay_fused_steps_kernel: nodes_qb, halved (down to 4)
+// while that leaves fewer CTAs than SMs, so short vectors still spread over
+// the whole GPU.
+int fused_qb(int n, int64_t nquads, int sms) {
+    int qb = nodes_qb(n);
+    while (qb > 4 && (nquads + qb - 1) / qb < sms) qb /= 2;
+    return qb;
+}
+
+template <int OBJ, int OPT>
+int launch_fused(const relay_handle* h, const ModelArgs& a, const FusedSteps& fs, cudaStream_t stream) {
+    int dev = 0;
+    const int sms = device_sms(&dev);
+    if (sms <= 0) return RELAY_ECUDA;
+    const int qb = fused_qb(h->prog.n, a.nquads, sms);
+    const int threads = qb * h->prog.n;
+    const size_t smem = static_cast<size_t>(2) * h->prog.E * qb * 16 + static_cast<size_t>(fs.k) * h->prog.n * 8;
+    if (smem > static_cast<size_t>(kMaxSmem)) return RELAY_EUNSUPPORTED;
+    const int per_sm = resident_ctas<relay_fused_steps_kernel<OBJ, OPT>>(dev, threads, smem);
+    if (per_sm <= 0) return RELAY_ECUDA;
+    const int64_t want = (a.nquads + qb - 1) / qb;
+    const int64_t cap = static_cast<int64_t>(sms) * per_sm;
+    const int grid = static_cast<int>(want < cap ? want : cap);
+    const PhiloxKey mu_key = philox_key(static_cast<uint64_t>(h->obj.k0) | (static_cast<uint64_t>(h->obj.k1) << 32));
+    relay_fused_steps_kernel<OBJ, OPT><<<grid, threads, smem, stream>>>(program_of(h), objective_of<OBJ>(h), mu_key, a, fs, qb);
+    return launch_status();
+}
+
+template <int OPT>
+int launch_fused_obj(const relay_handle* h, const ModelArgs& a, const FusedSteps& fs, cudaStream_t stream) {
+    if (h->obj.source == relaysum::kMuStored) return launch_fused<relaysum::kMuStored, OPT>(h, a, fs, stream);
+    return launch_fused<relaysum::kMuPerRow, OPT>(h, a, fs, stream);
+}
+
+// Window k of a counter launch: handle h's program, lost mask and arrays.
+template <int NT>
+void count_window(const relay_handle* h, int32_t* counts, CountWindows<NT>& cw, int k) {
+    cw.prog[k] = program_of(h);
+    std::memcpy(cw.lost[k].w, h->lost, sizeof(cw.lost[k].w));
+    cw.has_lost[k] = h->has_lost ? 1 : 0;
+    cw.counts[k] = counts;
+    cw.dme_count[k] = h->algo == RELAY_ALGO_DME ? h->dme_count : nullptr;
+}
+
+}  // namespace
+
+namespace relaysum {
+namespace RELAY_SPACE {
+
+int launch_counts(const relay_handle* const* hs, int32_t* const* counts, int windows, cudaStream_t stream) {
+    if (windows == 1) {
+        CountWindows<1> cw;
+        count_window(hs[0], counts[0], cw, 0);
+        relay_counts_kernel<1><<<1, 256, 0, stream>>>(cw);
+    } else {
+        CountWindows<2> cw;
+        for (int k = 0; k < 2; ++k) count_window(hs[k], counts[k], cw, k);
+        relay_counts_kernel<2><<<2, 256, 0, stream>>>(cw);
+    }
+    return launch_status();
+}
+
+int launch_step(const relay_handle* h, const ModelArgs& a, bool nodes, cudaStream_t stream, bool after_counts) {
+    switch (h->opt) {
+        case 0: return launch_models_obj<0>(h, a, nodes, stream, after_counts);
+        case 1: return launch_models_obj<1>(h, a, nodes, stream, after_counts);
+        default: return launch_models_obj<2>(h, a, nodes, stream, after_counts);
+    }
+}
+
+int launch_step_windows(const relay_handle* const* hs, const ModelArgs* as, cudaStream_t stream, bool after_counts) {
+    switch (hs[0]->opt) {
+        case 0: return launch_walk_obj<0, 2>(hs, as, stream, after_counts);
+        case 1: return launch_walk_obj<1, 2>(hs, as, stream, after_counts);
+        default: return launch_walk_obj<2, 2>(hs, as, stream, after_counts);
+    }
+}
+
+int launch_steps(const relay_handle* h, const ModelArgs& a, FusedSteps& fs, cudaStream_t stream) {
+    switch (h->opt) {
+        case 0: return launch_fused_obj<0>(h, a, fs, stream);
+        case 1: return launch_fused_obj<1>(h, a, fs, stream);
+        default: return launch_fused_obj<2>(h, a, fs, stream);
+    }
+}
+
+int launch_steps_counts(const relay_handle* h, int32_t* counts, int k, cudaStream_t stream) {
+    LostMask lost;
+    std::memcpy(lost.w, h->lost, sizeof(lost.w));
+    relay_counts_steps_kernel<<<1, kCountsThreads, 0, stream>>>(program_of(h), lost, h->has_lost ? 1 : 0, counts,
+                                                                h->algo == RELAY_ALGO_DME ? h->dme_count : nullptr, k);
+    return launch_status();
+}
+
+}  // namespace RELAY_SPACE
+}  // namespace relaysum

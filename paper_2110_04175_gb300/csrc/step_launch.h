@@ -1,0 +1,30 @@
+// step_launch.h -- the launches of step_kernels.cu, one set per capacity (the
+// namespaces), for the C ABI (relaysum.cu), which has checked the arguments.
+#pragma once
+
+namespace relaysum {
+namespace small {
+// The counter kernel over `windows` (1 or 2) handles.
+int launch_counts(const relay_handle* const* hs, int32_t* const* counts, int windows, cudaStream_t stream);
+// The step kernel (the node-parallel one or the walk); after_counts: as the
+// programmatic dependent of the counter kernel just enqueued.
+int launch_step(const relay_handle* h, const ModelArgs& a, bool nodes, cudaStream_t stream, bool after_counts);
+// The walk over two handles' windows.
+int launch_step_windows(const relay_handle* const* hs, const ModelArgs* as, cudaStream_t stream, bool after_counts);
+// Several steps in one launch, and the counters behind it.
+int launch_steps(const relay_handle* h, const ModelArgs& a, FusedSteps& fs, cudaStream_t stream);
+int launch_steps_counts(const relay_handle* h, int32_t* counts, int k, cudaStream_t stream);
+}  // namespace small
+namespace large {
+// The counter kernel over `windows` (1 or 2) handles.
+int launch_counts(const relay_handle* const* hs, int32_t* const* counts, int windows, cudaStream_t stream);
+// The step kernel (the node-parallel one or the walk); after_counts: as the
+// programmatic dependent of the counter kernel just enqueued.
+int launch_step(const relay_handle* h, const ModelArgs& a, bool nodes, cudaStream_t stream, bool after_counts);
+// The walk over two handles' windows.
+int launch_step_windows(const relay_handle* const* hs, const ModelArgs* as, cudaStream_t stream, bool after_counts);
+// Several steps in one launch, and the counters behind it.
+int launch_steps(const relay_handle* h, const ModelArgs& a, FusedSteps& fs, cudaStream_t stream);
+int launch_steps_counts(const relay_handle* h, int32_t* counts, int k, cudaStream_t stream);
+}  // namespace large
+}  // namespace relaysum
