@@ -94,16 +94,142 @@ PhiloxKey philox_key(uint64_t seed) {
 __device__ __forceinline__ uint4 philox4x32_10(uint4 c, const PhiloxKey& key) {
 #pragma unroll
     for (int round = 0; round < 10; ++round) {
-        const uint32_t hi0 = __umulhi(kPhiloxM0, c.x), lo0 = kPhiloxM0 * c.x;
-        const uint32_t hi1 = __umulhi(kPhiloxM1, c.z), lo1 = kPhiloxM1 * c.z;
-        c = make_uint4(hi1 ^ c.y ^ key.k[round][0], lo1, hi0 ^ c.w ^ key.k[round][1], lo0);
+        const uint64_t p0 = static_cast<uint64_t>(kPhiloxM0) * c.x, p1 = static_cast<uint64_t>(kPhiloxM1) * c.z;
+        c = make_uint4(static_cast<uint32_t>(p1 >> 32) ^ c.y ^ key.k[round][0], static_cast<uint32_t>(p1),
+                       static_cast<uint32_t>(p0 >> 32) ^ c.w ^ key.k[round][1], static_cast<uint32_t>(p0));
     }
     return c;
 }
 
-// 24 high bits -> (0, 1], exact in fp32.
-__device__ __forceinline__ float unit_interval(uint32_t w) {
-    return __uint2float_rn((w >> 8) + 1u) * 5.9604644775390625e-8f;  // 2^-24
+// The noise block of worker `row` at quad q in step `step` (stream 0),
+// philox4x32_10 of (q, row, step, 0) with its first two rounds split: what
+// depends on the quad alone is formed once per quad (NoiseQuad), what depends
+// on the row and the step not per quad, so 16 to 17 of the 20 wide products
+// remain per call.  They are what bounds the noise: a wide product holds the
+// heavy multiplier pipe for 4 cycles a warp.
+struct NoiseQuad {
+    uint32_t a, b, d;
+};
+
+__device__ __forceinline__ uint64_t wide_product(uint32_t m, uint32_t v) { return static_cast<uint64_t>(m) * v; }
+__device__ __forceinline__ uint32_t hi32(uint64_t p) { return static_cast<uint32_t>(p >> 32); }
+__device__ __forceinline__ uint32_t lo32(uint64_t p) { return static_cast<uint32_t>(p); }
+
+__device__ __forceinline__ NoiseQuad noise_quad(uint32_t q, const PhiloxKey& key) {
+    const uint64_t p0 = wide_product(kPhiloxM0, q);
+    const uint64_t p1 = wide_product(kPhiloxM1, hi32(p0) ^ key.k[0][1]);
+    return NoiseQuad{hi32(p1), lo32(p1), lo32(p0)};
+}
+
+__device__ __forceinline__ uint4 noise_words(const NoiseQuad& t, uint32_t row, uint32_t step, const PhiloxKey& key) {
+    const uint64_t ps = wide_product(kPhiloxM1, step);
+    const uint64_t pr = wide_product(kPhiloxM0, hi32(ps) ^ row ^ key.k[0][0]);
+    uint4 c = make_uint4(t.a ^ (lo32(ps) ^ key.k[1][0]), t.b, t.d ^ (hi32(pr) ^ key.k[1][1]), lo32(pr));
+#pragma unroll
+    for (int round = 2; round < 10; ++round) {
+        const uint64_t p0 = wide_product(kPhiloxM0, c.x), p1 = wide_product(kPhiloxM1, c.z);
+        c = make_uint4(hi32(p1) ^ c.y ^ key.k[round][0], lo32(p1), hi32(p0) ^ c.w ^ key.k[round][1], lo32(p0));
+    }
+    return c;
+}
+
+// ------------------------------------------------------- packed fp32 pairs
+
+// The step is bound by instruction issue wherever HBM does not bound it, and
+// sm_103a's packed fp32 instructions (add / mul / fma .rn.f32x2) do the work
+// of two scalar ones in one issue slot, each half rounded as the scalar one.
+// All per-coordinate arithmetic goes through these, and every fused
+// multiply-add is written out, so that every kernel rounds alike.
+struct Pair {
+    unsigned long long v;
+};
+
+__device__ __forceinline__ Pair pack(float lo, float hi) {
+    Pair r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ Pair pack(float both) { return pack(both, both); }
+__device__ __forceinline__ void unpack(Pair p, float& lo, float& hi) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(p.v));
+}
+__device__ __forceinline__ Pair add2(Pair a, Pair b) {
+    Pair r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ Pair mul2(Pair a, Pair b) {
+    Pair r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ Pair fma2(Pair a, Pair b, Pair c) {
+    Pair r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+    return r;
+}
+
+__device__ __forceinline__ float4 quad(Pair a, Pair b) {
+    float4 r;
+    unpack(a, r.x, r.y);
+    unpack(b, r.z, r.w);
+    return r;
+}
+__device__ __forceinline__ float4 add4(float4 a, float4 b) {
+    return quad(add2(pack(a.x, a.y), pack(b.x, b.y)), add2(pack(a.z, a.w), pack(b.z, b.w)));
+}
+// Products with one factor for the whole quad stay scalar: the factor can be
+// a constant operand, where a pair of it would cost two moves, and the scalar
+// multiplier pipe is otherwise idle (Philox fills the other one).  Each is
+// rounded once; the intrinsics keep a later add from being fused in (the
+// regenerated mu rounds exactly like the stored one).
+__device__ __forceinline__ float4 fma4(float w, float4 z, float4 acc) {  // w z + acc
+    return make_float4(__fmaf_rn(w, z.x, acc.x), __fmaf_rn(w, z.y, acc.y), __fmaf_rn(w, z.z, acc.z),
+                       __fmaf_rn(w, z.w, acc.w));
+}
+__device__ __forceinline__ float4 sub4(float4 a, float4 b) {
+    return make_float4(__fsub_rn(a.x, b.x), __fsub_rn(a.y, b.y), __fsub_rn(a.z, b.z), __fsub_rn(a.w, b.w));
+}
+__device__ __forceinline__ float4 scale4(float4 a, float s) {
+    return make_float4(__fmul_rn(a.x, s), __fmul_rn(a.y, s), __fmul_rn(a.z, s), __fmul_rn(a.w, s));
+}
+
+// ------------------------------------------------------------------ normals
+
+// u = ((w >> 8) + 1) 2^-24 in (0, 1] for two words: the 24-bit integers and
+// the product-sum are exact in fp32.
+__device__ __forceinline__ Pair unit_interval2(uint32_t w0, uint32_t w1) {
+    const Pair ulp = pack(5.9604644775390625e-8f);  // 2^-24
+    return fma2(pack(__uint2float_rn(w0 >> 8), __uint2float_rn(w1 >> 8)), ulp, ulp);
+}
+
+// -2 ln u for two u in [2^-24, 1].  u = m 2^e with m in [sqrt(1/2), sqrt(2));
+// with f = m - 1 (exact), -2 ln u = -2 ln 2 e + f P(f), and P, the minimax
+// polynomial of degree 8 of -2 ln(1 + f) / f with P(0) = -2 (fitted by the
+// Remez exchange for the relative error of the result, 2.0e-8, coefficients
+// rounded one by one), keeps the relative accuracy where u is just below 1
+// and ln u next to 0.  Over all 2^24 values of u: the radius sqrt(-2 ln u) is
+// within 1.4e-7 of the exact one (rms 2.1e-8; a correctly rounded logarithm
+// gives 1.2e-7 and 1.8e-8), far inside what the sine and cosine leave.
+__device__ __forceinline__ Pair minus_2_ln(Pair u) {
+    float u0, u1;
+    unpack(u, u0, u1);
+    const int b0 = __float_as_int(u0), b1 = __float_as_int(u1);
+    const int e0 = (b0 - 0x3f3504f3) & static_cast<int>(0xff800000u);  // e 2^23
+    const int e1 = (b1 - 0x3f3504f3) & static_cast<int>(0xff800000u);
+    const Pair f = add2(pack(__int_as_float(b0 - e0), __int_as_float(b1 - e1)), pack(-1.0f));
+    Pair p = pack(-0.18646626f);
+    p = fma2(p, f, pack(0.29618296f));
+    p = fma2(p, f, pack(-0.29821008f));
+    p = fma2(p, f, pack(0.32977396f));
+    p = fma2(p, f, pack(-0.39912102f));
+    p = fma2(p, f, pack(0.5001276f));
+    p = fma2(p, f, pack(-0.66668445f));
+    p = fma2(p, f, pack(0.99999815f));
+    p = fma2(p, f, pack(-2.0f));
+    // -2 ln 2 e, e as the integer e 2^23
+    const Pair c = pack(-1.38629436111989061883f * 1.1920928955078125e-7f);
+    return fma2(pack(__int2float_rn(e0), __int2float_rn(e1)), c, mul2(f, p));
 }
 
 __device__ __forceinline__ float sqrt_approx(float v) {
@@ -111,44 +237,51 @@ __device__ __forceinline__ float sqrt_approx(float v) {
     asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
     return r;
 }
+__device__ __forceinline__ float sin_approx(float v) {
+    float r;
+    asm("sin.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
+    return r;
+}
+__device__ __forceinline__ float cos_approx(float v) {
+    float r;
+    asm("cos.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
+    return r;
+}
 
-// Four standard normals for coordinates 4q .. 4q+3 (Box-Muller on the two
-// word pairs of one Philox block): z = sqrt(-2 ln u_a) (cos, sin)(2 pi u_b).
+// The gradient noise: MINUS four standard normals for coordinates 4q .. 4q+3
+// (Box-Muller on the two word pairs of one Philox block): z = sqrt(-2 ln u_a) (cos, sin)(2 pi u_b).
 // The angle is taken as 2 pi u_b - pi, inside the range where the hardware
-// sine/cosine are accurate to 2^-21.4, and the half turn is undone by the
-// sign; the radius keeps an accurate logarithm (its argument can sit just
-// below 1, where an approximate one loses all relative accuracy).
+// sine/cosine are accurate to 2^-21.4; the half turn flips the sign, which the
+// callers put into their factor (an exact step that costs nothing there).
+__device__ __forceinline__ float4 minus_normal4(uint4 w) {
+    float l0, l1, t0, t1;
+    unpack(minus_2_ln(unit_interval2(w.x, w.z)), l0, l1);
+    constexpr float kTwoPi = 6.28318530717958647692f, kPi = 3.14159265358979323846f;
+    unpack(fma2(unit_interval2(w.y, w.w), pack(kTwoPi), pack(-kPi)), t0, t1);
+    return quad(mul2(pack(sqrt_approx(l0)), pack(cos_approx(t0), sin_approx(t0))),
+                mul2(pack(sqrt_approx(l1)), pack(cos_approx(t1), sin_approx(t1))));
+}
+
+// Four standard normals of the centres (stream 1) and of the initial model
+// (stream 2): the same words and angles with CUDA's logf and __sincosf.  These
+// are the objective that a run is defined by, read back through
+// relay_fill_objective and relay_metrics in double, so they keep their bits.
 __device__ __forceinline__ float4 normal4(uint32_t q, uint32_t row, uint32_t step, uint32_t stream,
                                           const PhiloxKey& key) {
     const uint4 w = philox4x32_10(make_uint4(q, row, step, stream), key);
-    const float r0 = sqrt_approx(-2.0f * logf(unit_interval(w.x)));
-    const float r1 = sqrt_approx(-2.0f * logf(unit_interval(w.z)));
+    float u0, u1, t0, t1;
+    unpack(unit_interval2(w.x, w.z), u0, u1);
     constexpr float kTwoPi = 6.28318530717958647692f, kPi = 3.14159265358979323846f;
+    unpack(fma2(unit_interval2(w.y, w.w), pack(kTwoPi), pack(-kPi)), t0, t1);
+    const float r0 = sqrt_approx(-2.0f * logf(u0)), r1 = sqrt_approx(-2.0f * logf(u1));
     float s0, c0, s1, c1;
-    __sincosf(fmaf(unit_interval(w.y), kTwoPi, -kPi), &s0, &c0);
-    __sincosf(fmaf(unit_interval(w.w), kTwoPi, -kPi), &s1, &c1);
+    __sincosf(t0, &s0, &c0);
+    __sincosf(t1, &s1, &c1);
     return make_float4(-r0 * c0, -r0 * s0, -r1 * c1, -r1 * s1);
 }
 
-// ------------------------------------------------------------ float4 helpers
+// ------------------------------------------------------------ float4 access
 
-__device__ __forceinline__ float4 add4(float4 a, float4 b) {
-    return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
-}
-__device__ __forceinline__ float4 sub4(float4 a, float4 b) {
-    return make_float4(a.x - b.x, a.y - b.y, a.z - b.z, a.w - b.w);
-}
-__device__ __forceinline__ float4 scale4(float4 a, float s) {
-    return make_float4(a.x * s, a.y * s, a.z * s, a.w * s);
-}
-// Rounded product that the compiler may not fuse into a later add: the
-// regenerated mu must round exactly like the stored one.
-__device__ __forceinline__ float4 scale4_rn(float4 a, float s) {
-    return make_float4(__fmul_rn(a.x, s), __fmul_rn(a.y, s), __fmul_rn(a.z, s), __fmul_rn(a.w, s));
-}
-__device__ __forceinline__ float4 fma4(float w, float4 z, float4 acc) {
-    return make_float4(fmaf(w, z.x, acc.x), fmaf(w, z.y, acc.y), fmaf(w, z.z, acc.z), fmaf(w, z.w, acc.w));
-}
 // Loads read once per step: read-only path, no L1 allocation.
 __device__ __forceinline__ float4 ld_stream(const float* p) {
     float4 v;
@@ -188,7 +321,7 @@ __device__ __forceinline__ float4 centre(const Obj& obj, const PhiloxKey& mu_key
                                  : cen[obj.col[j] * cen_stride];
             acc = fma4(obj.w[j], z, acc);
         }
-        return scale4_rn(acc, obj.scale);
+        return scale4(acc, obj.scale);
     }
 }
 

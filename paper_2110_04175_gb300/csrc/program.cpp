@@ -211,13 +211,17 @@ int assign_slots(const Tree& t, const Walk& w, int root, bool received_sums, Pro
         tot[i] = (wide && m > 0) ? alloc() : -1;
         rsum[i] = (wide && m > 0 && received_sums) ? alloc() : -1;
         p->rsum_slot[i] = static_cast<int8_t>(rsum[i]);
-        int parent_pos = -1;
+        // i's neighbours in the order in which its rebuild adds their
+        // messages: the DFS parent's at i's visit, then each child's at the
+        // child's visit
+        const int parent_pos = par >= 0 ? 0 : -1;
         for (int s = 0; s < D; ++s) {
-            const int k = t.nbr[i][s];
+            const int k = (s == parent_pos) ? par : w.children[i][s - (parent_pos + 1)];
             const int pos = pos_base[i] + s;
-            p->pos_in[pos] = static_cast<int16_t>(t.in_edge[i][s]);
-            p->pos_out[pos] = static_cast<int16_t>(t.out_edge[i][s]);
-            if (k == par) parent_pos = s;
+            const auto& l = t.nbr[i];
+            const size_t at = std::lower_bound(l.begin(), l.end(), k) - l.begin();
+            p->pos_in[pos] = static_cast<int16_t>(t.in_edge[i][at]);
+            p->pos_out[pos] = static_cast<int16_t>(t.out_edge[i][at]);
             int slot = -1;
             if (k != par) {
                 if (wide) {
@@ -247,18 +251,6 @@ int assign_slots(const Tree& t, const Walk& w, int root, bool received_sums, Pro
             release(rsum[par]);
         }
         p->order[v] = static_cast<int16_t>(i);
-    }
-    // rebuild order of every worker's incoming messages: the walk adds the
-    // DFS parent's message at the worker's visit, then each child's at the
-    // child's visit
-    auto in_from = [&](int i, int k) {
-        const auto& l = t.nbr[i];
-        return t.in_edge[i][std::lower_bound(l.begin(), l.end(), k) - l.begin()];
-    };
-    for (int i = 0; i < n; ++i) {
-        int k = pos_base[i];
-        if (w.parent[i] >= 0) p->rb_in[k++] = static_cast<int16_t>(in_from(i, w.parent[i]));
-        for (int c : w.children[i]) p->rb_in[k++] = static_cast<int16_t>(in_from(i, c));
     }
     (void)root;
     return next_id;
@@ -313,7 +305,6 @@ void narrow(const Program& from, SmallProgram* to) {
     std::copy_n(from.pos_slot, from.E, to->pos_slot);
     std::copy_n(from.edge_src, from.E, to->edge_src);
     std::copy_n(from.edge_dst, from.E, to->edge_dst);
-    std::copy_n(from.rb_in, from.E, to->rb_in);
     std::copy_n(from.rsum_slot, from.n, to->rsum_slot);
     std::copy_n(from.rsum_row, from.n, to->rsum_row);
 }

@@ -33,8 +33,9 @@
 //
 // The same program drives the node-parallel kernel for short vectors (one
 // thread per worker and quad): it forms each worker's messages with the
-// walk's arithmetic and adds the incoming ones in the walk's order (rb_in),
-// so both kernels give the same bits.
+// walk's arithmetic and adds the incoming ones in the walk's order (a worker's
+// positions are in that order: its DFS parent, then its children as they are
+// visited), so both kernels give the same bits.
 //
 // The program is a plain-old-data struct passed by value as a
 // __grid_constant__ kernel parameter (warp-uniform reads from the constant
@@ -55,7 +56,7 @@ enum NodeFlags : int16_t {
 
 struct NodeRec {        // 20 bytes; indexed by worker id
     int16_t deg;        // D = |N(i)|
-    int16_t pos_base;   // first of i's D positions (ascending neighbour id)
+    int16_t pos_base;   // first of i's D positions (the DFS parent, then the children in visit order)
     int16_t parent_pos; // position of the DFS parent among i's neighbours; -1 at the root
     int16_t recv_slot;  // slot holding m^t_{parent->i} (or T_parent); -1 at the root
     int16_t acc_slot;   // slot of i's rebuild accumulator; -1 for a leaf
@@ -78,9 +79,6 @@ struct ProgramT {
     int16_t pos_slot[kE];     // narrow node: slot of the message to child k_s; else -1
     int16_t edge_src[kE];     // directed edge e: edge_src[e] -> edge_dst[e]
     int16_t edge_dst[kE];
-    int16_t rb_in[kE];        // i's positions: its incoming edges in the walk's rebuild
-                                 // order (from the DFS parent, then from the children in
-                                 // visit order); the node-parallel kernel adds them so
     // received sums (built only when they are on; else -1): a wide node's
     // slot of its running sum S_i^t, and its row among the sum rows (row
     // E + rsum_row[i] of a message buffer).  int8 keeps two programs within

@@ -67,7 +67,7 @@ __global__ void relay_fill_mu_kernel(float* mu, const float* mix, int n, int K, 
                     acc = fma4(w, z, acc);
                 }
             }
-            const float4 sv = scale4_rn(acc, scale);
+            const float4 sv = scale4(acc, scale);
             *reinterpret_cast<float4*>(mu + i * ld_x + c) =
                 make_float4(sv.x, c + 1 < d ? sv.y : 0.f, c + 2 < d ? sv.z : 0.f, c + 3 < d ? sv.w : 0.f);
         }
@@ -736,7 +736,7 @@ int relay_program(const relay_handle* h, int32_t* nslots, int32_t* order, int32_
             pos_rec[4 * e] = p.pos_in[e];
             pos_rec[4 * e + 1] = p.pos_out[e];
             pos_rec[4 * e + 2] = p.pos_slot[e];
-            pos_rec[4 * e + 3] = p.rb_in[e];
+            pos_rec[4 * e + 3] = p.pos_in[e];
         }
     return RELAY_OK;
 }

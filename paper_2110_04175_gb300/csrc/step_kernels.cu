@@ -258,27 +258,26 @@ __device__ __noinline__ void visit_wide(const Program& prog, const NodeRec& r, c
 //   Adam:     m = beta1 m + (1 - beta1) g;  v = beta2 v + (1 - beta2) g^2;
 //             u = -adam_step m / (sqrt(v) adam_ibc2 + eps)     (s1 = m, s2 = v)
 // The rule on the optimiser state (m, v) held in registers; adam_step and
-// adam_ibc2 are the factors of this step.
+// adam_ibc2 are the factors of this step.  Returns u for Adam, and the
+// direction u / -lr otherwise (relayed_with applies -lr).
 template <int OPT>
 __device__ __forceinline__ float4 update_rule(const ModelArgs& a, float adam_step, float adam_ibc2, float4 g,
                                               float4& m, float4& v) {
-    if (OPT == 0) return scale4(g, -a.lr);
+    if (OPT == 0) return g;
     if (OPT == 1) {
-        m = make_float4(fmaf(a.beta1, m.x, g.x), fmaf(a.beta1, m.y, g.y), fmaf(a.beta1, m.z, g.z),
-                        fmaf(a.beta1, m.w, g.w));
-        return make_float4(-a.lr * fmaf(a.beta1, m.x, g.x), -a.lr * fmaf(a.beta1, m.y, g.y),
-                           -a.lr * fmaf(a.beta1, m.z, g.z), -a.lr * fmaf(a.beta1, m.w, g.w));
+        m = fma4(a.beta1, m, g);
+        return fma4(a.beta1, m, g);
     }
     const float c1 = 1.0f - a.beta1, c2 = 1.0f - a.beta2;
-    m = make_float4(fmaf(a.beta1, m.x, c1 * g.x), fmaf(a.beta1, m.y, c1 * g.y), fmaf(a.beta1, m.z, c1 * g.z),
-                    fmaf(a.beta1, m.w, c1 * g.w));
-    v = make_float4(fmaf(a.beta2, v.x, c2 * g.x * g.x), fmaf(a.beta2, v.y, c2 * g.y * g.y),
-                    fmaf(a.beta2, v.z, c2 * g.z * g.z), fmaf(a.beta2, v.w, c2 * g.w * g.w));
+    m = fma4(a.beta1, m, scale4(g, c1));
+    const float4 cg = scale4(g, c2);
+    const float4 gg = quad(mul2(pack(cg.x, cg.y), pack(g.x, g.y)), mul2(pack(cg.z, cg.w), pack(g.z, g.w)));
+    v = fma4(a.beta2, v, gg);
     auto upd = [&](float mm, float vv) { return -adam_step * mm / fmaf(sqrtf(vv), adam_ibc2, a.eps); };
     return make_float4(upd(m.x, v.x), upd(m.y, v.y), upd(m.z, v.z), upd(m.w, v.w));
 }
 
-// One step's update with the state read from and written back to HBM.
+// One step's direction (or update) with the state read from and written back to HBM.
 template <int OPT>
 __device__ __forceinline__ float4 local_update(const ModelArgs& a, int i, int64_t q, float4 g) {
     float4 m = make_float4(0.f, 0.f, 0.f, 0.f), v = m;
@@ -287,10 +286,10 @@ __device__ __forceinline__ float4 local_update(const ModelArgs& a, int i, int64_
     float4* pv = reinterpret_cast<float4*>(a.s2 + i * a.ld_x + 4 * q);
     m = *pm;
     if (OPT == 2) v = *pv;
-    const float4 u = update_rule<OPT>(a, a.adam_step, a.adam_ibc2, g, m, v);
+    const float4 dir = update_rule<OPT>(a, a.adam_step, a.adam_ibc2, g, m, v);
     __stcs(pm, m);
     if (OPT == 2) __stcs(pv, v);
-    return u;
+    return dir;
 }
 
 // Per-worker rebuild factors from this step's counters: x' = scale * acc
@@ -326,24 +325,21 @@ __device__ __forceinline__ void rebuild_factors(const Program& prog, const Model
 
 // The relayed value of worker i at quad q: x^{t+1/2} = x + u (Alg. 1), the
 // update u (Alg. 6) or the sample mu + sigma xi (Alg. 5), with
-// g = (x - mu) + sigma xi and z the worker's noise normals.
-// `update` maps g to u (and advances the optimiser state).
-template <typename Update>
+// g = (x - mu) + sigma xi and z MINUS the worker's noise normals.
+// `update` maps g to the optimiser's direction (and advances its state).
+template <int OPT, typename Update>
 __device__ __forceinline__ float4 relayed_with(const ModelArgs& a, float4 xv, float4 mv, float4 z,
                                                Update update) {
-    if (a.algo == 2)
-        return make_float4(fmaf(a.sigma, z.x, mv.x), fmaf(a.sigma, z.y, mv.y), fmaf(a.sigma, z.z, mv.z),
-                           fmaf(a.sigma, z.w, mv.w));
-    const float4 g = make_float4(fmaf(a.sigma, z.x, xv.x - mv.x), fmaf(a.sigma, z.y, xv.y - mv.y),
-                                 fmaf(a.sigma, z.z, xv.z - mv.z), fmaf(a.sigma, z.w, xv.w - mv.w));
-    const float4 u = update(g);
-    return (a.algo == 1) ? u : add4(xv, u);
+    if (a.algo == 2) return fma4(-a.sigma, z, mv);
+    const float4 dir = update(fma4(-a.sigma, z, sub4(xv, mv)));
+    if (OPT == 2) return (a.algo == 1) ? dir : add4(xv, dir);
+    return (a.algo == 1) ? scale4(dir, -a.lr) : fma4(-a.lr, dir, xv);
 }
 
 template <int OPT>
 __device__ __forceinline__ float4 relayed_value(const ModelArgs& a, int i, int64_t q, float4 xv, float4 mv,
                                                 float4 z) {
-    return relayed_with(a, xv, mv, z, [&](float4 g) { return local_update<OPT>(a, i, q, g); });
+    return relayed_with<OPT>(a, xv, mv, z, [&](float4 g) { return local_update<OPT>(a, i, q, g); });
 }
 
 // The step of NT handles in one launch: one handle, or the tree windows of
@@ -390,6 +386,7 @@ __device__ __forceinline__ void walk(const Program& prog, const ModelArgs& a, co
             for (int k = 0; k < obj.K; ++k)
                 cen[k * blockDim.x] = normal4(a.q0 + static_cast<uint32_t>(q), static_cast<uint32_t>(k), 0u, 1u, mu_key);
     }
+    const NoiseQuad nq = noise_quad(a.q0 + static_cast<uint32_t>(q), a.key);
     wait_for_prior_grid();
     rebuild_factors(prog, a, s_scale, s_fill);
     __syncthreads();
@@ -414,13 +411,12 @@ __device__ __forceinline__ void walk(const Program& prog, const ModelArgs& a, co
             const float* mp = a.msg_in + prog.pos_out[r.pos_base + r.parent_pos] * a.ld_m + 4 * q;
             back = a.rsum ? ld_stream(mp) : __ldg(reinterpret_cast<const float4*>(mp));
         }
-        const float4 z = normal4(a.q0 + static_cast<uint32_t>(q), static_cast<uint32_t>(i),
-                                 a.step, 0u, a.key);
+        const float4 z = minus_normal4(noise_words(nq, static_cast<uint32_t>(i), a.step, a.key));
         const float4 xh = relayed_value<OPT>(a, i, q, xv, mv, z);
         // the rebuild sum starts from fill_i x_i (robust rule: n - nbar_i;
         // Alg. 6: n; Alg. 5: 1; Alg. 1: nothing)
         float4 acc = xh;
-        if (s_fill[i] != 0.0f) acc = add4(scale4(xv, s_fill[i]), xh);
+        if (s_fill[i] != 0.0f) acc = fma4(s_fill[i], xv, xh);
         float4 recv = make_float4(0.f, 0.f, 0.f, 0.f);
         if (r.recv_slot >= 0) {
             recv = sl[r.recv_slot];
@@ -591,8 +587,8 @@ relay_nodes_kernel(const __grid_constant__ Program prog, const __grid_constant__
         float4 xh = make_float4(0.f, 0.f, 0.f, 0.f);
         if (active) {
             const float4 mv = (OBJ == relaysum::kMuStored) ? ms : centre<kObj>(obj, mu_key, a, i, q, nullptr, 0);
-            const float4 z = normal4(a.q0 + static_cast<uint32_t>(q), static_cast<uint32_t>(i), a.step, 0u,
-                                     a.key);
+            const float4 z = minus_normal4(noise_words(noise_quad(a.q0 + static_cast<uint32_t>(q), a.key),
+                                                       static_cast<uint32_t>(i), a.step, a.key));
             xh = relayed_value<OPT>(a, i, q, xv, mv, z);
             switch (r.deg) {
                 case 0: break;
@@ -612,17 +608,17 @@ relay_nodes_kernel(const __grid_constant__ Program prog, const __grid_constant__
         if (active) {
             // the rebuild sum starts from fill_i x_i + x^{t+1/2}, as in the walk
             float4 acc = xh;
-            if (s_fill[i] != 0.0f) acc = add4(scale4(xv, s_fill[i]), xh);
+            if (s_fill[i] != 0.0f) acc = fma4(s_fill[i], xv, xh);
             if (a.rsum && r.deg > kRegDeg) {  // and the wide node's received sum S_i^t, in the same order
                 float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
                 for (int k = 0; k < r.deg; ++k) {
-                    const float4 m = m_new[prog.rb_in[r.pos_base + k] * qb];
+                    const float4 m = m_new[prog.pos_in[r.pos_base + k] * qb];
                     acc = add4(acc, m);
                     sum = add4(sum, m);
                 }
                 st_stream(a.msg_out + rsum_row(prog, i) * a.ld_m + 4 * q, sum);
             } else {
-                for (int k = 0; k < r.deg; ++k) acc = add4(acc, m_new[prog.rb_in[r.pos_base + k] * qb]);
+                for (int k = 0; k < r.deg; ++k) acc = add4(acc, m_new[prog.pos_in[r.pos_base + k] * qb]);
             }
             st_stream(a.x + i * a.ld_x + 4 * q, scale4(acc, s_scale[i]));
         }
@@ -675,7 +671,7 @@ template <int D>
 __device__ __forceinline__ float4 fused_rebuild(const Program& prog, const NodeRec& r, const float4* cur, int qb,
                                                 float4 acc) {
 #pragma unroll
-    for (int k = 0; k < D; ++k) acc = add4(acc, cur[prog.rb_in[r.pos_base + k] * qb]);
+    for (int k = 0; k < D; ++k) acc = add4(acc, cur[prog.pos_in[r.pos_base + k] * qb]);
     return acc;
 }
 
@@ -747,6 +743,7 @@ relay_fused_steps_kernel(const __grid_constant__ Program prog, const __grid_cons
             const int64_t qg = b * qb + (idx - e * qb);
             fused_mem[E * qb + idx] = qg < a.nquads ? ld_stream(a.msg_in + e * a.ld_m + 4 * qg) : zero;
         }
+        const NoiseQuad nq = noise_quad(a.q0 + static_cast<uint32_t>(q), a.key);
         float4 xv = zero, mv = zero, m1 = zero, m2 = zero;
         if (active) {
             xv = *reinterpret_cast<const float4*>(a.x + i * a.ld_x + 4 * q);
@@ -761,10 +758,10 @@ relay_fused_steps_kernel(const __grid_constant__ Program prog, const __grid_cons
             const float4* const prev = fused_mem + ((j + 1) & 1) * E * qb + qi;
             float4 xh = zero;
             if (active) {
-                const float4 z = normal4(a.q0 + static_cast<uint32_t>(q), static_cast<uint32_t>(i),
-                                         a.step + static_cast<uint32_t>(j), 0u, a.key);
+                const float4 z = minus_normal4(noise_words(nq, static_cast<uint32_t>(i),
+                                                           a.step + static_cast<uint32_t>(j), a.key));
                 const float st = fs.adam_step[j], ib = fs.adam_ibc2[j];
-                xh = relayed_with(a, xv, mv, z, [&](float4 g) { return update_rule<OPT>(a, st, ib, g, m1, m2); });
+                xh = relayed_with<OPT>(a, xv, mv, z, [&](float4 g) { return update_rule<OPT>(a, st, ib, g, m1, m2); });
                 float* const out = (E > 0 && j + 2 >= fs.k) ? fs.msg[(j + 1) & 1] + 4 * q : nullptr;
                 switch (r.deg) {
                     case 0: break;
@@ -779,7 +776,7 @@ relay_fused_steps_kernel(const __grid_constant__ Program prog, const __grid_cons
             if (active) {
                 const float2 f = factors[j * n + i];  // (scale, fill)
                 float4 acc = xh;
-                if (f.y != 0.0f) acc = add4(scale4(xv, f.y), xh);
+                if (f.y != 0.0f) acc = fma4(f.y, xv, xh);
                 switch (r.deg) {
                     case 0: break;
                     case 1: acc = fused_rebuild<1>(prog, r, cur, qb, acc); break;
@@ -787,7 +784,7 @@ relay_fused_steps_kernel(const __grid_constant__ Program prog, const __grid_cons
                     case 3: acc = fused_rebuild<3>(prog, r, cur, qb, acc); break;
                     case 4: acc = fused_rebuild<4>(prog, r, cur, qb, acc); break;
                     default:
-                        for (int k = 0; k < r.deg; ++k) acc = add4(acc, cur[prog.rb_in[r.pos_base + k] * qb]);
+                        for (int k = 0; k < r.deg; ++k) acc = add4(acc, cur[prog.pos_in[r.pos_base + k] * qb]);
                         break;
                 }
                 xv = scale4(acc, f.x);
