@@ -55,6 +55,8 @@ constexpr int kMaxFusedSteps = 64;  // steps per launch (Adam's per-step factors
 
 struct FusedSteps {
     int32_t k;                        // steps in this launch, 1 .. kMaxFusedSteps
+    int32_t rounds;                   // counter rounds until they repeat, 1 .. k (settled_rounds)
+    int32_t qb_log2;                  // quads per CTA
     float* msg[2];                    // step t0 + j reads msg[j & 1] and writes msg[(j + 1) & 1]
     float adam_step[kMaxFusedSteps];  // Adam's factors of step t0 + j
     float adam_ibc2[kMaxFusedSteps];

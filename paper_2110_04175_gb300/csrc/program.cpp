@@ -17,6 +17,7 @@
 #include <cstring>
 #include <functional>
 #include <queue>
+#include <utility>
 #include <vector>
 
 #include "relaysum.h"
@@ -87,6 +88,22 @@ int validate(int n, const int32_t* edges, int n_edges, Tree* t, Program* p) {
     }
     return RELAY_OK;
 }
+
+// The farthest worker from `from`, and its distance in edges.
+std::pair<int, int> farthest(const Tree& t, int from) {
+    std::vector<int> dist(t.n, -1), bfs{from};
+    dist[from] = 0;
+    for (size_t q = 0; q < bfs.size(); ++q)
+        for (int j : t.nbr[bfs[q]])
+            if (dist[j] < 0) {
+                dist[j] = dist[bfs[q]] + 1;
+                bfs.push_back(j);
+            }
+    return {bfs.back(), dist[bfs.back()]};
+}
+
+// Edges of the longest path: from the worker farthest from any one.
+int diameter(const Tree& t) { return farthest(t, farthest(t, 0).first).second; }
 
 // A walk from one root: parent, children in visit order, pre-order.
 struct Walk {
@@ -222,6 +239,7 @@ int assign_slots(const Tree& t, const Walk& w, int root, bool received_sums, Pro
             const size_t at = std::lower_bound(l.begin(), l.end(), k) - l.begin();
             p->pos_in[pos] = static_cast<int16_t>(t.in_edge[i][at]);
             p->pos_out[pos] = static_cast<int16_t>(t.out_edge[i][at]);
+            p->edge_pos[t.in_edge[i][at]] = static_cast<int16_t>(pos);
             int slot = -1;
             if (k != par) {
                 if (wide) {
@@ -286,6 +304,10 @@ int build_program(int n, const int32_t* edges, int n_edges, Program* out, bool r
     const Walk w = make_walk(t, best_root, received_sums);
     out->nslots = assign_slots(t, w, best_root, received_sums, out);
     out->root = best_root;
+    for (int i = 0; i < n; ++i) out->by_degree[i] = static_cast<uint8_t>(i);
+    std::stable_sort(out->by_degree, out->by_degree + n,
+                     [&](uint8_t a, uint8_t b) { return out->node[a].deg < out->node[b].deg; });
+    out->diameter = diameter(t);
     // a received-sum slot must fit its int8 field
     if (received_sums && out->nwide > 0 && out->nslots > 127) return RELAY_EUNSUPPORTED;
     return RELAY_OK;
@@ -298,6 +320,7 @@ void narrow(const Program& from, SmallProgram* to) {
     to->nslots = from.nslots;
     to->root = from.root;
     to->nwide = from.nwide;
+    to->diameter = from.diameter;
     std::copy_n(from.order, from.n, to->order);
     std::copy_n(from.node, from.n, to->node);
     std::copy_n(from.pos_in, from.E, to->pos_in);
@@ -305,6 +328,8 @@ void narrow(const Program& from, SmallProgram* to) {
     std::copy_n(from.pos_slot, from.E, to->pos_slot);
     std::copy_n(from.edge_src, from.E, to->edge_src);
     std::copy_n(from.edge_dst, from.E, to->edge_dst);
+    std::copy_n(from.edge_pos, from.E, to->edge_pos);
+    std::copy_n(from.by_degree, from.n, to->by_degree);
     std::copy_n(from.rsum_slot, from.n, to->rsum_slot);
     std::copy_n(from.rsum_row, from.n, to->rsum_row);
 }

@@ -79,6 +79,9 @@ struct ProgramT {
     int16_t pos_slot[kE];     // narrow node: slot of the message to child k_s; else -1
     int16_t edge_src[kE];     // directed edge e: edge_src[e] -> edge_dst[e]
     int16_t edge_dst[kE];
+    int16_t edge_pos[kE];     // directed edge e: the position at which it arrives (pos_in's inverse)
+    uint8_t by_degree[kN];    // the workers in ascending degree
+    int32_t diameter;            // edges of the tree's longest path
     // received sums (built only when they are on; else -1): a wide node's
     // slot of its running sum S_i^t, and its row among the sum rows (row
     // E + rsum_row[i] of a message buffer).  int8 keeps two programs within

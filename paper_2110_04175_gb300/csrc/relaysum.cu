@@ -696,8 +696,8 @@ int relay_steps(relay_handle* h, float* x, float* msg_a, float* msg_b, int32_t* 
         }
         // the counters advance after the models kernel, which read them
         if (counted) {
-            rc = is_small(h) ? relaysum::small::launch_steps_counts(h, counts, kc, stream)
-                             : relaysum::large::launch_steps_counts(h, counts, kc, stream);
+            rc = is_small(h) ? relaysum::small::launch_steps_counts(h, counts, kc, stream, h->d > 0)
+                             : relaysum::large::launch_steps_counts(h, counts, kc, stream, h->d > 0);
             if (rc != RELAY_OK) return rc;
         }
         done += kc;

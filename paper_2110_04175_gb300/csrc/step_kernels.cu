@@ -113,23 +113,36 @@ __global__ void relay_counts_kernel(const __grid_constant__ CountWindows<NT> cw)
     }
 }
 
+// Rounds of the counter recurrence after which it repeats: the counter of
+// edge i -> j depends on c^{-1} only through edges one hop further from j, so
+// after as many rounds as the tree's longest path has edges it is a function
+// of the tree and the lost messages alone, and every later round gives it
+// again.  A call of k steps needs no more rounds than that, whatever the
+// counters it starts from.
+int settled_rounds(const Program& prog, int64_t k) {
+    const int64_t d = prog.diameter > 1 ? prog.diameter : 1;
+    return static_cast<int>(k < d ? k : d);
+}
+
 // The counters (and the mean-estimation counts) advanced by k steps, for
 // relay_steps: one CTA of kCountsThreads >= n threads (thread i carries
-// worker i's mean-estimation count), the counters of the two step parities
-// in shared memory, one barrier per step.
+// worker i's mean-estimation count), the counters of the two round parities
+// in shared memory, one barrier per round.  Launched as a programmatic
+// dependent of the models kernel, which reads the same counters and writes
+// none: the rounds run beside it, and only the writes wait for it.
 constexpr int kCountsThreads = 256;
 static_assert(kMaxN <= kCountsThreads, "relay_counts_steps_kernel gives each worker its own thread");
 
 __global__ void __launch_bounds__(kCountsThreads)
 relay_counts_steps_kernel(const __grid_constant__ Program prog,
                                           const __grid_constant__ LostMask lost, int has_lost, int32_t* counts,
-                                          int64_t* dme_count, int k) {
+                                          int64_t* dme_count, int k, int rounds) {
     __shared__ int32_t c[2][kMaxE];
     const int E = prog.E;
     for (int e = threadIdx.x; e < E; e += blockDim.x) c[1][e] = counts[e];
     __syncthreads();
     int64_t received = 0;  // worker threadIdx.x: sum over the k steps of 1 + sum_j c^t_{j->i}
-    for (int j = 0; j < k; ++j) {
+    for (int j = 0; j < rounds; ++j) {
         const int32_t* c_old = c[(j + 1) & 1];
         int32_t* c_new = c[j & 1];
         for (int e = threadIdx.x; e < E; e += blockDim.x) c_new[e] = next_count(prog, lost, has_lost, c_old, e);
@@ -138,10 +151,11 @@ relay_counts_steps_kernel(const __grid_constant__ Program prog,
             const NodeRec r = prog.node[threadIdx.x];
             int64_t nb = 1;
             for (int p = 0; p < r.deg; ++p) nb += c_new[prog.pos_in[r.pos_base + p]];
-            received += nb;
+            received += (j + 1 == rounds) ? nb * (k - j) : nb;  // the last round's counters stay
         }
     }
-    for (int e = threadIdx.x; e < E; e += blockDim.x) counts[e] = c[(k - 1) & 1][e];
+    wait_for_prior_grid();
+    for (int e = threadIdx.x; e < E; e += blockDim.x) counts[e] = c[(rounds - 1) & 1][e];
     if (dme_count && threadIdx.x < prog.n) dme_count[threadIdx.x] += received;
 }
 
@@ -327,19 +341,20 @@ __device__ __forceinline__ void rebuild_factors(const Program& prog, const Model
 // update u (Alg. 6) or the sample mu + sigma xi (Alg. 5), with
 // g = (x - mu) + sigma xi and z MINUS the worker's noise normals.
 // `update` maps g to the optimiser's direction (and advances its state).
-template <int OPT, typename Update>
+// PLAIN: the caller knows that the algorithm is Alg. 1.
+template <int OPT, bool PLAIN, typename Update>
 __device__ __forceinline__ float4 relayed_with(const ModelArgs& a, float4 xv, float4 mv, float4 z,
                                                Update update) {
-    if (a.algo == 2) return fma4(-a.sigma, z, mv);
+    if (!PLAIN && a.algo == 2) return fma4(-a.sigma, z, mv);
     const float4 dir = update(fma4(-a.sigma, z, sub4(xv, mv)));
-    if (OPT == 2) return (a.algo == 1) ? dir : add4(xv, dir);
-    return (a.algo == 1) ? scale4(dir, -a.lr) : fma4(-a.lr, dir, xv);
+    if (!PLAIN && a.algo == 1) return (OPT == 2) ? dir : scale4(dir, -a.lr);
+    return (OPT == 2) ? add4(xv, dir) : fma4(-a.lr, dir, xv);
 }
 
 template <int OPT>
 __device__ __forceinline__ float4 relayed_value(const ModelArgs& a, int i, int64_t q, float4 xv, float4 mv,
                                                 float4 z) {
-    return relayed_with<OPT>(a, xv, mv, z, [&](float4 g) { return local_update<OPT>(a, i, q, g); });
+    return relayed_with<OPT, false>(a, xv, mv, z, [&](float4 g) { return local_update<OPT>(a, i, q, g); });
 }
 
 // The step of NT handles in one launch: one handle, or the tree windows of
@@ -627,99 +642,206 @@ relay_nodes_kernel(const __grid_constant__ Program prog, const __grid_constant__
 
 // ------------------------------------------------ several steps per launch
 
-// relay_steps: k consecutive steps in one launch, in the node-parallel
-// layout.  Every coordinate evolves on its own (the counters are the same
-// for all of them), so a CTA carries its qb quads of every worker through
-// all k steps without hearing from another CTA: models, centres and
-// optimiser state stay in registers, the messages of the step just taken
-// in shared memory, and the CTA advances its own copy of the counters.  HBM
-// is read once (x, mu, the optimiser state, m^{t0-1}) and written once (x,
-// the state, and the messages of the last two steps, which k relay_step
-// calls leave in the two buffers).  Each step is the node kernel's
-// arithmetic in the node kernel's order, so the result equals k relay_step
-// calls bit for bit.
-// Outgoing messages of worker i from its incoming ones in shared memory
-// (`prev`, this thread's column), with node_small's / node_wide's arithmetic.
-// They go to `cur`, and to HBM at `out` (row e at out + e * ld_m) unless null.
-template <int D>
-__device__ __forceinline__ void fused_small(const Program& prog, const NodeRec& r, const ModelArgs& a, float4 xh,
-                                            const float4* prev, float4* cur, int qb, float* out,
-                                            uint32_t lost_bits) {
-    float4 m[D];
-#pragma unroll
-    for (int s = 0; s < D; ++s) m[s] = prev[prog.pos_in[r.pos_base + s] * qb];
-    float4 pre[D];
-    pre[0] = xh;
-#pragma unroll
-    for (int s = 1; s < D; ++s) pre[s] = add4(pre[s - 1], m[s - 1]);
-    float4 suf[D];
-    suf[D - 1] = m[D - 1];
-#pragma unroll
-    for (int s = D - 2; s >= 0; --s) suf[s] = add4(m[s], suf[s + 1]);
+// relay_steps: k consecutive steps in one launch, one thread per (worker,
+// quad).  Every coordinate evolves on its own (the counters are the same for
+// all of them), so a CTA carries its qb quads of every worker through all k
+// steps without hearing from another CTA: models, centres, optimiser state
+// and the messages that arrived last stay in registers, and the messages of
+// the step being taken pass through shared memory.  HBM is read once (x, mu,
+// the optimiser state, m^{t0-1}) and written once (x, the state, and the
+// messages of the last two steps, which k relay_step calls leave in the two
+// buffers).  Each step is the node kernel's arithmetic in the node kernel's
+// order, so the result equals k relay_step calls bit for bit.
+// The CTA's step barrier (barrier 1): its warps may reach it at different
+// places in the code, one per number of neighbours.
+__device__ __forceinline__ void cta_barrier() { asm volatile("bar.sync 1, %0;" ::"r"(blockDim.x) : "memory"); }
+
+// What a thread of relay_fused_steps_kernel is: one worker's share of one
+// quad at a time.
+struct FusedThread {
+    int i, deg;            // worker (deg 0 on the threads that fill up the last warp)
+    int pos_base;          // its first position
+    int in;                // float4 index of its first incoming message in a buffer; the next is qb further
+    uint32_t lost_bits;    // bit s: its message to neighbour s is lost (narrow nodes)
+};
+
+// One launch's k steps of one quad for a warp whose workers all have at most
+// D neighbours (D <= kRegDeg; a lane with fewer skips the missing ones).
+// The messages that arrived at the step before are registers m: they are read
+// from shared memory once, for the rebuild, and serve the next step's
+// outgoing messages from there.  One barrier per step: a buffer is written
+// again two steps later, when every thread has passed the barrier between,
+// that is finished reading it.  The next step's noise, which depends on
+// nothing here, is drawn between the loads of the new messages and their use.
+template <int D, int OPT, bool PLAIN>
+__device__ __forceinline__ void fused_steps(const Program& prog, const ModelArgs& a, const FusedSteps& fs,
+                                            const FusedThread& t, const float2* factors, float4* buf, int buf_len,
+                                            int qb, int& parity, bool active, int64_t q, float4& xv, float4 mv,
+                                            float4& m1, float4& m2) {
+    constexpr int DN = D > 0 ? D : 1;
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    float4 m[DN];
+    int out[DN];
 #pragma unroll
     for (int s = 0; s < D; ++s) {
-        const int e = prog.pos_out[r.pos_base + s];
-        const float4 o = ((lost_bits >> s) & 1u) ? make_float4(0.f, 0.f, 0.f, 0.f)
-                                                 : ((s == D - 1) ? pre[s] : add4(pre[s], suf[s + 1]));
-        cur[e * qb] = o;
-        if (out) st_stream(out + e * a.ld_m, o);
+        m[s] = zero;
+        out[s] = 0;
+        if (s < t.deg) {
+            // where the message to neighbour s arrives
+            out[s] = prog.edge_pos[prog.pos_out[t.pos_base + s]] * qb + (t.in - t.pos_base * qb);
+            if (active) m[s] = ld_stream(a.msg_in + prog.pos_in[t.pos_base + s] * a.ld_m + 4 * q);
+        }
+    }
+    const NoiseQuad nq = noise_quad(a.q0 + static_cast<uint32_t>(q), a.key);
+    const uint32_t row = static_cast<uint32_t>(t.i);
+    float4 z = minus_normal4(noise_words(nq, row, a.step, a.key));
+    float2 f = make_float2(0.f, 0.f);
+    for (int j = 0; j < fs.k; ++j) {
+        const float st = (OPT == 2) ? fs.adam_step[j] : 0.0f, ib = (OPT == 2) ? fs.adam_ibc2[j] : 0.0f;
+        const float4 xh =
+            relayed_with<OPT, PLAIN>(a, xv, mv, z, [&](float4 g) { return update_rule<OPT>(a, st, ib, g, m1, m2); });
+        if (D > 0 && j + 1 == fs.k && j > 0 && active) {  // m^{t0+k-2}, before it is replaced
+#pragma unroll
+            for (int s = 0; s < D; ++s)
+                if (s < t.deg)
+                    st_stream(fs.msg[j & 1] + prog.pos_in[t.pos_base + s] * a.ld_m + 4 * q, m[s]);
+        }
+        float4* const cur = buf + (parity ? buf_len : 0);
+        parity ^= 1;
+        if (D > 0) {
+            // outgoing message s = prefix(s) + suffix(s + 1), as node_small
+            float4 o[DN];
+            float4 pre = xh;
+            float4 suf[DN];
+            suf[DN - 1] = m[DN - 1];
+#pragma unroll
+            for (int s = D - 2; s >= 1; --s) suf[s] = add4(m[s], suf[s + 1]);
+#pragma unroll
+            for (int s = 0; s < D; ++s) {
+                // the zeros of a lane's missing neighbours add nothing
+                o[s] = (s == D - 1) ? pre : add4(pre, suf[s + 1]);
+                if (s + 1 < D) pre = add4(pre, m[s]);
+            }
+            if (t.lost_bits) {
+#pragma unroll
+                for (int s = 0; s < D; ++s)
+                    if ((t.lost_bits >> s) & 1u) o[s] = zero;
+            }
+#pragma unroll
+            for (int s = 0; s < D; ++s)
+                if (s < t.deg) cur[out[s]] = o[s];
+        }
+        cta_barrier();
+        if (D > 0) {
+#pragma unroll
+            for (int s = 0; s < D; ++s)
+                if (s < t.deg) m[s] = cur[t.in + s * qb];
+        }
+        if (j < fs.rounds) f = factors[j * prog.n + t.i];  // (scale, fill)
+        z = minus_normal4(noise_words(nq, row, a.step + static_cast<uint32_t>(j) + 1u, a.key));
+        float4 acc = xh;
+        if (f.y != 0.0f) acc = fma4(f.y, xv, acc);
+#pragma unroll
+        for (int s = 0; s < D; ++s) acc = add4(acc, m[s]);
+        xv = scale4(acc, f.x);
+    }
+    if (D > 0 && active) {
+        float* const last = fs.msg[fs.k & 1];
+#pragma unroll
+        for (int s = 0; s < D; ++s)
+            if (s < t.deg) st_stream(last + prog.pos_in[t.pos_base + s] * a.ld_m + 4 * q, m[s]);
     }
 }
 
-// The rebuild sum: acc plus the incoming messages of step j in rb_in order.
-template <int D>
-__device__ __forceinline__ float4 fused_rebuild(const Program& prog, const NodeRec& r, const float4* cur, int qb,
-                                                float4 acc) {
-#pragma unroll
-    for (int k = 0; k < D; ++k) acc = add4(acc, cur[prog.pos_in[r.pos_base + k] * qb]);
-    return acc;
-}
-
-__device__ __noinline__ void fused_wide(const Program& prog, const NodeRec& r, const ModelArgs& a, float4 xh,
-                                        const float4* prev, float4* cur, int qb, float* out) {
-    const int D = r.deg;
-    const int base = r.pos_base;
-    float4 total = xh;
-    for (int s = D - 1; s >= 0; --s) total = add4(total, prev[prog.pos_in[base + s] * qb]);
-    for (int s = 0; s < D; ++s) {
-        const int e = prog.pos_out[base + s];
-        const float4 o = delivered(a, e, sub4(total, prev[prog.pos_in[base + s] * qb]));
-        cur[e * qb] = o;
-        if (out) st_stream(out + e * a.ld_m, o);
+// The same for a warp with a worker of degree > kRegDeg (a star's hub): the
+// messages that arrived at the step before stay in shared memory, in the
+// worker's own rows of the other buffer, and the outgoing ones are formed as
+// node_small and node_wide form them.
+template <int OPT>
+__device__ __noinline__ void fused_steps_wide(const Program& prog, const ModelArgs& a, const FusedSteps& fs,
+                                              const FusedThread& t, const float2* factors, float4* buf, int buf_len,
+                                              int qb, int& parity, bool active, int64_t q, float4& xv, float4 mv,
+                                              float4& m1, float4& m2) {
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    const int qi = t.in - t.pos_base * qb;
+    const NoiseQuad nq = noise_quad(a.q0 + static_cast<uint32_t>(q), a.key);
+    float4* const first = buf + (parity ? 0 : buf_len) + t.in;
+    for (int s = 0; s < t.deg; ++s)
+        first[s * qb] = active ? ld_stream(a.msg_in + prog.pos_in[t.pos_base + s] * a.ld_m + 4 * q) : zero;
+    for (int j = 0; j < fs.k; ++j) {
+        float4* const cur = buf + (parity ? buf_len : 0);
+        const float4* const prev = buf + (parity ? 0 : buf_len) + t.in;
+        parity ^= 1;
+        const float4 z = minus_normal4(noise_words(nq, static_cast<uint32_t>(t.i), a.step + static_cast<uint32_t>(j),
+                                                   a.key));
+        const float4 xh = relayed_with<OPT, false>(a, xv, mv, z, [&](float4 g) {
+            return update_rule<OPT>(a, fs.adam_step[j], fs.adam_ibc2[j], g, m1, m2);
+        });
+        if (j + 1 == fs.k && j > 0 && active)  // m^{t0+k-2}
+            for (int s = 0; s < t.deg; ++s)
+                st_stream(fs.msg[j & 1] + prog.pos_in[t.pos_base + s] * a.ld_m + 4 * q, prev[s * qb]);
+        float4 total = xh;
+        if (t.deg > kRegDeg)
+            for (int s = t.deg - 1; s >= 0; --s) total = add4(total, prev[s * qb]);
+        for (int s = 0; s < t.deg; ++s) {
+            float4 o;
+            if (t.deg > kRegDeg) {
+                o = sub4(total, prev[s * qb]);
+            } else {
+                float4 pre = xh;
+                for (int r = 0; r < s; ++r) pre = add4(pre, prev[r * qb]);
+                o = pre;
+                if (s + 1 < t.deg) {
+                    float4 suf = prev[(t.deg - 1) * qb];
+                    for (int r = t.deg - 2; r > s; --r) suf = add4(prev[r * qb], suf);
+                    o = add4(pre, suf);
+                }
+            }
+            const int e = prog.pos_out[t.pos_base + s];
+            cur[prog.edge_pos[e] * qb + qi] = delivered(a, e, o);
+        }
+        cta_barrier();
+        const float2 f = factors[min(j, fs.rounds - 1) * prog.n + t.i];
+        float4 acc = xh;
+        if (f.y != 0.0f) acc = fma4(f.y, xv, xh);
+        for (int s = 0; s < t.deg; ++s) acc = add4(acc, cur[t.in + s * qb]);
+        xv = scale4(acc, f.x);
+    }
+    if (active) {
+        const float4* const last = buf + (parity ? 0 : buf_len) + t.in;
+        for (int s = 0; s < t.deg; ++s)
+            st_stream(fs.msg[fs.k & 1] + prog.pos_in[t.pos_base + s] * a.ld_m + 4 * q, last[s * qb]);
     }
 }
 
-// blockDim.x = qb * n <= 1024, threads worker-major as in relay_nodes_kernel.
-// Dynamic shared memory: two [E][qb] float4 message buffers, buffer j & 1
-// holding the messages of step t0 + j (buffer 1 starts with m^{t0-1}), then
-// the rebuild factors (scale, fill) of every worker and step, [k][n] float2.
-// The counters, hence the factors, are the same for every quad: the CTA
-// advances them through the k steps once, before its first quads.  One
-// barrier per step: a thread can write a buffer again only two steps later,
-// after every thread has passed the barrier between, i.e. finished reading it.
-template <int OBJ, int OPT>
-__global__ void __launch_bounds__(1024)
+// blockDim.x = qb * n rounded up to whole warps, at most kFusedThreads; qb
+// consecutive threads share a worker, the workers in ascending degree, so
+// that the workers of one warp have (nearly) the same number of neighbours
+// and no lane waits for another's longer code path.  Dynamic shared memory:
+// two [E][qb] float4 message buffers, row p holding the message that arrives
+// at position p (so a worker reads consecutive rows), then the rebuild
+// factors (scale, fill) of every worker and counter round, [rounds][n]
+// float2.  The counters, hence the factors, are the same for every quad: the
+// CTA advances them once, before its first quads.
+constexpr int kFusedThreads = 512;
+
+template <int OBJ, int OPT, bool PLAIN>
+__global__ void __launch_bounds__(kFusedThreads, 2)
 relay_fused_steps_kernel(const __grid_constant__ Program prog, const __grid_constant__ ObjectiveArg<OBJ> obj,
                          const __grid_constant__ PhiloxKey mu_key, const __grid_constant__ ModelArgs a,
-                         const __grid_constant__ FusedSteps fs, int qb) {
+                         const __grid_constant__ FusedSteps fs) {
+    allow_dependent_launch();  // the counter kernel behind this one waits for all of it before it writes
     extern __shared__ float4 fused_mem[];
-    __shared__ int32_t c_mem[2][kMaxE];  // counters of the step parities
+    __shared__ int32_t c_mem[2][kMaxE];  // counters of the round parities
     constexpr int kObj = (OBJ == relaysum::kMuStored) ? relaysum::kMuStored : relaysum::kMuPerRow;
     const int tid = static_cast<int>(threadIdx.x);
-    const int i = tid / qb;
-    const int qi = tid - i * qb;
+    const int qb = 1 << fs.qb_log2;
     const int n = prog.n;
     const int E = prog.E;
-    const NodeRec r = prog.node[i];
-    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-    float2* const factors = reinterpret_cast<float2*>(fused_mem + 2 * E * qb);  // [j * n + i]
-    // bit s: the message to this worker's neighbour s is lost (narrow nodes)
-    uint32_t lost_bits = 0;
-    if (a.has_lost && r.deg <= kRegDeg)
-        for (int s = 0; s < r.deg; ++s) lost_bits |= (a.lost(prog.pos_out[r.pos_base + s]) ? 1u : 0u) << s;
+    float2* const factors = reinterpret_cast<float2*>(fused_mem + 2 * E * qb);  // [round * n + i]
     for (int e = tid; e < E; e += blockDim.x) c_mem[1][e] = a.counts[e];  // c^{t0-1}
     __syncthreads();
-    for (int j = 0; j < fs.k; ++j) {
+    for (int j = 0; j < fs.rounds; ++j) {
         const int32_t* const c_old = c_mem[(j + 1) & 1];
         int32_t* const c_new = c_mem[j & 1];
         for (int e = tid; e < E; e += blockDim.x) c_new[e] = next_count(prog, a.lost, a.has_lost, c_old, e);
@@ -733,69 +855,52 @@ relay_fused_steps_kernel(const __grid_constant__ Program prog, const __grid_cons
             factors[j * n + w] = make_float2(scale, fill);
         }
     }
-    const int64_t nblk = (a.nquads + qb - 1) / qb;
+    __syncthreads();
+    const int slot = tid >> fs.qb_log2;
+    const int qi = tid & (qb - 1);
+    const bool live = slot < n;
+    FusedThread t;
+    t.i = prog.by_degree[live ? slot : n - 1];
+    t.deg = live ? prog.node[t.i].deg : 0;
+    t.pos_base = live ? prog.node[t.i].pos_base : 0;
+    t.in = t.pos_base * qb + qi;
+    t.lost_bits = 0;
+    if (a.has_lost && t.deg <= kRegDeg)
+        for (int s = 0; s < t.deg; ++s) t.lost_bits |= (a.lost(prog.pos_out[t.pos_base + s]) ? 1u : 0u) << s;
+    const int widest = __reduce_max_sync(0xffffffffu, t.deg);
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    const int64_t nblk = (a.nquads + qb - 1) >> fs.qb_log2;
+    int parity = 0;
     for (int64_t b = blockIdx.x; b < nblk; b += gridDim.x) {
-        const int64_t q = b * qb + qi;
-        const bool active = q < a.nquads;
-        // m^{t0-1} of this CTA's quads (coalesced rows of qb quads) into buffer 1
-        for (int idx = tid; idx < E * qb; idx += blockDim.x) {
-            const int e = idx / qb;
-            const int64_t qg = b * qb + (idx - e * qb);
-            fused_mem[E * qb + idx] = qg < a.nquads ? ld_stream(a.msg_in + e * a.ld_m + 4 * qg) : zero;
-        }
-        const NoiseQuad nq = noise_quad(a.q0 + static_cast<uint32_t>(q), a.key);
+        const int64_t q = (b << fs.qb_log2) + qi;
+        const bool active = live && q < a.nquads;
         float4 xv = zero, mv = zero, m1 = zero, m2 = zero;
         if (active) {
-            xv = *reinterpret_cast<const float4*>(a.x + i * a.ld_x + 4 * q);
-            mv = (OBJ == relaysum::kMuStored) ? ld_stream(a.mu + i * a.ld_x + 4 * q)
-                                               : centre<kObj>(obj, mu_key, a, i, q, nullptr, 0);
-            if (OPT >= 1) m1 = *reinterpret_cast<const float4*>(a.s1 + i * a.ld_x + 4 * q);
-            if (OPT == 2) m2 = *reinterpret_cast<const float4*>(a.s2 + i * a.ld_x + 4 * q);
+            xv = *reinterpret_cast<const float4*>(a.x + t.i * a.ld_x + 4 * q);
+            mv = (OBJ == relaysum::kMuStored) ? ld_stream(a.mu + t.i * a.ld_x + 4 * q)
+                                               : centre<kObj>(obj, mu_key, a, t.i, q, nullptr, 0);
+            if (OPT >= 1) m1 = *reinterpret_cast<const float4*>(a.s1 + t.i * a.ld_x + 4 * q);
+            if (OPT == 2) m2 = *reinterpret_cast<const float4*>(a.s2 + t.i * a.ld_x + 4 * q);
         }
-        __syncthreads();
-        for (int j = 0; j < fs.k; ++j) {
-            float4* const cur = fused_mem + (j & 1) * E * qb + qi;
-            const float4* const prev = fused_mem + ((j + 1) & 1) * E * qb + qi;
-            float4 xh = zero;
-            if (active) {
-                const float4 z = minus_normal4(noise_words(nq, static_cast<uint32_t>(i),
-                                                           a.step + static_cast<uint32_t>(j), a.key));
-                const float st = fs.adam_step[j], ib = fs.adam_ibc2[j];
-                xh = relayed_with<OPT>(a, xv, mv, z, [&](float4 g) { return update_rule<OPT>(a, st, ib, g, m1, m2); });
-                float* const out = (E > 0 && j + 2 >= fs.k) ? fs.msg[(j + 1) & 1] + 4 * q : nullptr;
-                switch (r.deg) {
-                    case 0: break;
-                    case 1: fused_small<1>(prog, r, a, xh, prev, cur, qb, out, lost_bits); break;
-                    case 2: fused_small<2>(prog, r, a, xh, prev, cur, qb, out, lost_bits); break;
-                    case 3: fused_small<3>(prog, r, a, xh, prev, cur, qb, out, lost_bits); break;
-                    case 4: fused_small<4>(prog, r, a, xh, prev, cur, qb, out, lost_bits); break;
-                    default: fused_wide(prog, r, a, xh, prev, cur, qb, out); break;
-                }
-            }
-            __syncthreads();
-            if (active) {
-                const float2 f = factors[j * n + i];  // (scale, fill)
-                float4 acc = xh;
-                if (f.y != 0.0f) acc = fma4(f.y, xv, xh);
-                switch (r.deg) {
-                    case 0: break;
-                    case 1: acc = fused_rebuild<1>(prog, r, cur, qb, acc); break;
-                    case 2: acc = fused_rebuild<2>(prog, r, cur, qb, acc); break;
-                    case 3: acc = fused_rebuild<3>(prog, r, cur, qb, acc); break;
-                    case 4: acc = fused_rebuild<4>(prog, r, cur, qb, acc); break;
-                    default:
-                        for (int k = 0; k < r.deg; ++k) acc = add4(acc, cur[prog.pos_in[r.pos_base + k] * qb]);
-                        break;
-                }
-                xv = scale4(acc, f.x);
-            }
+        switch (widest) {
+#define RELAY_FUSED(D) \
+    fused_steps<D, OPT, PLAIN>(prog, a, fs, t, factors, fused_mem, E * qb, qb, parity, active, q, xv, mv, m1, m2)
+            case 0: RELAY_FUSED(0); break;
+            case 1: RELAY_FUSED(1); break;
+            case 2: RELAY_FUSED(2); break;
+            case 3: RELAY_FUSED(3); break;
+            case 4: RELAY_FUSED(4); break;
+#undef RELAY_FUSED
+            default:
+                fused_steps_wide<OPT>(prog, a, fs, t, factors, fused_mem, E * qb, qb, parity, active, q, xv, mv, m1,
+                                      m2);
+                break;
         }
         if (active) {
-            st_stream(a.x + i * a.ld_x + 4 * q, xv);
-            if (OPT >= 1) st_stream(a.s1 + i * a.ld_x + 4 * q, m1);
-            if (OPT == 2) st_stream(a.s2 + i * a.ld_x + 4 * q, m2);
+            st_stream(a.x + t.i * a.ld_x + 4 * q, xv);
+            if (OPT >= 1) st_stream(a.s1 + t.i * a.ld_x + 4 * q, m1);
+            if (OPT == 2) st_stream(a.s2 + t.i * a.ld_x + 4 * q, m2);
         }
-        __syncthreads();  // the next block refills buffer 1
     }
 }
 
@@ -996,38 +1101,45 @@ int launch_models_obj(const relay_handle* h, const ModelArgs& a, bool nodes, cud
     return launch_walk_obj<OPT, 1>(&h, &a, stream, after_counts);
 }
 
-// Quads per CTA of relay_fused_steps_kernel: nodes_qb, halved (down to 4)
-// while that leaves fewer CTAs than SMs, so short vectors still spread over
-// the whole GPU.
-int fused_qb(int n, int64_t nquads, int sms) {
-    int qb = nodes_qb(n);
-    while (qb > 4 && (nquads + qb - 1) / qb < sms) qb /= 2;
-    return qb;
+// Quads per CTA of relay_fused_steps_kernel (as a power of two): as many as
+// fill kFusedThreads, at most a warp's worth, halved while that leaves fewer
+// CTAs than SMs (short vectors then still spread over the whole GPU) and the
+// CTA keeps a full warp.
+int fused_qb_log2(int n, int64_t nquads, int sms) {
+    int l = 5;
+    while (l > 0 && (n << l) > kFusedThreads) --l;
+    while (l > 0 && (n << (l - 1)) >= 32 && (nquads + (int64_t(1) << l) - 1) >> l < sms) --l;
+    return l;
 }
 
-template <int OBJ, int OPT>
-int launch_fused(const relay_handle* h, const ModelArgs& a, const FusedSteps& fs, cudaStream_t stream) {
+template <int OBJ, int OPT, bool PLAIN>
+int launch_fused(const relay_handle* h, const ModelArgs& a, FusedSteps& fs, cudaStream_t stream) {
     int dev = 0;
     const int sms = device_sms(&dev);
     if (sms <= 0) return RELAY_ECUDA;
-    const int qb = fused_qb(h->prog.n, a.nquads, sms);
-    const int threads = qb * h->prog.n;
-    const size_t smem = static_cast<size_t>(2) * h->prog.E * qb * 16 + static_cast<size_t>(fs.k) * h->prog.n * 8;
+    const int n = h->prog.n;
+    fs.qb_log2 = fused_qb_log2(n, a.nquads, sms);
+    const int threads = ((n << fs.qb_log2) + 31) / 32 * 32;
+    const size_t smem = (static_cast<size_t>(2) * h->prog.E << fs.qb_log2) * 16 + static_cast<size_t>(fs.rounds) * n * 8;
     if (smem > static_cast<size_t>(kMaxSmem)) return RELAY_EUNSUPPORTED;
-    const int per_sm = resident_ctas<relay_fused_steps_kernel<OBJ, OPT>>(dev, threads, smem);
+    const int per_sm = resident_ctas<relay_fused_steps_kernel<OBJ, OPT, PLAIN>>(dev, threads, smem);
     if (per_sm <= 0) return RELAY_ECUDA;
-    const int64_t want = (a.nquads + qb - 1) / qb;
+    const int64_t want = (a.nquads + (int64_t(1) << fs.qb_log2) - 1) >> fs.qb_log2;
     const int64_t cap = static_cast<int64_t>(sms) * per_sm;
     const int grid = static_cast<int>(want < cap ? want : cap);
     const PhiloxKey mu_key = philox_key(static_cast<uint64_t>(h->obj.k0) | (static_cast<uint64_t>(h->obj.k1) << 32));
-    relay_fused_steps_kernel<OBJ, OPT><<<grid, threads, smem, stream>>>(program_of(h), objective_of<OBJ>(h), mu_key, a, fs, qb);
+    relay_fused_steps_kernel<OBJ, OPT, PLAIN><<<grid, threads, smem, stream>>>(program_of(h), objective_of<OBJ>(h), mu_key, a, fs);
     return launch_status();
 }
 
 template <int OPT>
-int launch_fused_obj(const relay_handle* h, const ModelArgs& a, const FusedSteps& fs, cudaStream_t stream) {
-    if (h->obj.source == relaysum::kMuStored) return launch_fused<relaysum::kMuStored, OPT>(h, a, fs, stream);
-    return launch_fused<relaysum::kMuPerRow, OPT>(h, a, fs, stream);
+int launch_fused_obj(const relay_handle* h, const ModelArgs& a, FusedSteps& fs, cudaStream_t stream) {
+    const bool plain = h->algo == RELAY_ALGO_RELAYSGD;
+    if (h->obj.source == relaysum::kMuStored)
+        return plain ? launch_fused<relaysum::kMuStored, OPT, true>(h, a, fs, stream)
+                     : launch_fused<relaysum::kMuStored, OPT, false>(h, a, fs, stream);
+    return plain ? launch_fused<relaysum::kMuPerRow, OPT, true>(h, a, fs, stream)
+                 : launch_fused<relaysum::kMuPerRow, OPT, false>(h, a, fs, stream);
 }
 
 // Window k of a counter launch: handle h's program, lost mask and arrays.
@@ -1075,6 +1187,7 @@ int launch_step_windows(const relay_handle* const* hs, const ModelArgs* as, cuda
 }
 
 int launch_steps(const relay_handle* h, const ModelArgs& a, FusedSteps& fs, cudaStream_t stream) {
+    fs.rounds = settled_rounds(program_of(h), fs.k);
     switch (h->opt) {
         case 0: return launch_fused_obj<0>(h, a, fs, stream);
         case 1: return launch_fused_obj<1>(h, a, fs, stream);
@@ -1082,12 +1195,14 @@ int launch_steps(const relay_handle* h, const ModelArgs& a, FusedSteps& fs, cuda
     }
 }
 
-int launch_steps_counts(const relay_handle* h, int32_t* counts, int k, cudaStream_t stream) {
+int launch_steps_counts(const relay_handle* h, int32_t* counts, int k, cudaStream_t stream, bool after_models) {
     LostMask lost;
     std::memcpy(lost.w, h->lost, sizeof(lost.w));
-    relay_counts_steps_kernel<<<1, kCountsThreads, 0, stream>>>(program_of(h), lost, h->has_lost ? 1 : 0, counts,
-                                                                h->algo == RELAY_ALGO_DME ? h->dme_count : nullptr, k);
-    return launch_status();
+    const auto& prog = program_of(h);
+    return launch_step_kernel(relay_counts_steps_kernel, 1, kCountsThreads, 0, stream, after_models, prog, lost,
+                              h->has_lost ? 1 : 0, counts,
+                              h->algo == RELAY_ALGO_DME ? h->dme_count : static_cast<int64_t*>(nullptr), k,
+                              settled_rounds(prog, k));
 }
 
 }  // namespace RELAY_SPACE

@@ -13,7 +13,7 @@ int launch_step(const relay_handle* h, const ModelArgs& a, bool nodes, cudaStrea
 int launch_step_windows(const relay_handle* const* hs, const ModelArgs* as, cudaStream_t stream, bool after_counts);
 // Several steps in one launch, and the counters behind it.
 int launch_steps(const relay_handle* h, const ModelArgs& a, FusedSteps& fs, cudaStream_t stream);
-int launch_steps_counts(const relay_handle* h, int32_t* counts, int k, cudaStream_t stream);
+int launch_steps_counts(const relay_handle* h, int32_t* counts, int k, cudaStream_t stream, bool after_models);
 }  // namespace small
 namespace large {
 // The counter kernel over `windows` (1 or 2) handles.
@@ -25,6 +25,6 @@ int launch_step(const relay_handle* h, const ModelArgs& a, bool nodes, cudaStrea
 int launch_step_windows(const relay_handle* const* hs, const ModelArgs* as, cudaStream_t stream, bool after_counts);
 // Several steps in one launch, and the counters behind it.
 int launch_steps(const relay_handle* h, const ModelArgs& a, FusedSteps& fs, cudaStream_t stream);
-int launch_steps_counts(const relay_handle* h, int32_t* counts, int k, cudaStream_t stream);
+int launch_steps_counts(const relay_handle* h, int32_t* counts, int k, cudaStream_t stream, bool after_models);
 }  // namespace large
 }  // namespace relaysum
