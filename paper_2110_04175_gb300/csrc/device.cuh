@@ -171,6 +171,9 @@ __device__ __forceinline__ Pair fma2(Pair a, Pair b, Pair c) {
     return r;
 }
 
+// a - b (the product with -1 is exact)
+__device__ __forceinline__ Pair sub2(Pair a, Pair b) { return fma2(b, pack(-1.0f), a); }
+
 __device__ __forceinline__ float4 quad(Pair a, Pair b) {
     float4 r;
     unpack(a, r.x, r.y);
@@ -307,6 +310,18 @@ __device__ __forceinline__ void st_stream(float* p, float4 v) {
     __stcs(reinterpret_cast<float4*>(p), v);
 }
 
+// ------------------------------------------------- programmatic dependent launch
+
+// relay_step launches the step kernel as a programmatic dependent of the
+// counter kernel: the counter kernel lets it be scheduled at once, and the
+// step kernel waits for the counter kernel's completion (and its writes)
+// before its first read of the counters.  Launched the ordinary way, the
+// wait returns immediately.
+__device__ __forceinline__ void allow_dependent_launch() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void wait_for_prior_grid() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // mu_i for quad q: read, or regenerated exactly as relay_fill_mu_kernel
 // writes it (same normals, same fma order), so both sources give the same bits.
 template <int OBJ, typename Obj>
@@ -348,6 +363,69 @@ int device_sms(int* dev_out) {
 
 int launch_status() {
     return cudaGetLastError() == cudaSuccess ? RELAY_OK : RELAY_ECUDA;
+}
+
+// Launches a step kernel; `after_counts` makes it a programmatic dependent of
+// the counter kernel just enqueued on the same stream (relay_step only).
+template <typename... Params, typename... Args>
+int launch_step_kernel(void (*kernel)(Params...), int grid, int threads, size_t smem, cudaStream_t stream,
+                       bool after_counts, Args... args) {
+    if (!after_counts) {
+        kernel<<<grid, threads, smem, stream>>>(args...);
+        return launch_status();
+    }
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(static_cast<unsigned>(grid));
+    cfg.blockDim = dim3(static_cast<unsigned>(threads));
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (cudaLaunchKernelEx(&cfg, kernel, args...) != cudaSuccess) return RELAY_ECUDA;
+    return launch_status();
+}
+
+// Opts `Kernel` in to the dynamic shared memory it may use (kMaxSmem, less
+// when its static shared memory and kMaxSmem would pass the device's per-CTA
+// limit) once per device, and returns its resident CTAs per SM for
+// (threads, smem).  Both are cached per device (queried once, not per step:
+// steps may be captured into CUDA graphs); each kernel instantiation has its
+// own cache.  0 on a CUDA error, which is cleared so that it is not reported
+// again by a later launch.
+template <auto Kernel>
+int resident_ctas(int dev, int threads, size_t smem) {
+    static std::atomic<bool> smem_set[kMaxDevices];
+    if (dev >= kMaxDevices || !smem_set[dev].load()) {
+        cudaFuncAttributes fa;
+        int optin = 0;
+        if (cudaFuncGetAttributes(&fa, Kernel) != cudaSuccess ||
+            cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) {
+            (void)cudaGetLastError();
+            return 0;
+        }
+        const int room = optin - static_cast<int>(fa.sharedSizeBytes);
+        if (room <= 0 ||
+            cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 room < kMaxSmem ? room : kMaxSmem) != cudaSuccess) {
+            (void)cudaGetLastError();
+            return 0;
+        }
+        if (dev < kMaxDevices) smem_set[dev].store(true);
+    }
+    static std::atomic<int64_t> occ_cache[kMaxDevices];
+    const int64_t key = static_cast<int64_t>(smem) * 1024 + threads;
+    const int64_t cached = dev < kMaxDevices ? occ_cache[dev].load() : 0;
+    if (cached != 0 && (cached >> 8) == key) return static_cast<int>(cached & 0xFF);
+    int per_sm = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, Kernel, threads, smem) != cudaSuccess || per_sm <= 0) {
+        (void)cudaGetLastError();
+        return 0;
+    }
+    if (dev < kMaxDevices) occ_cache[dev].store((key << 8) | (per_sm & 0xFF));
+    return per_sm;
 }
 
 }  // namespace

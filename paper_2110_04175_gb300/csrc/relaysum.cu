@@ -82,33 +82,32 @@ __global__ void relay_fill_mu_kernel(float* mu, const float* mix, int n, int K, 
 //   xi   += sum_i (x_i - xbar)^2        dist += (xbar - mubar)^2
 // Pass 1: each block reduces its share of the coordinates (grid-stride,
 // fixed order) into partials[2 blockIdx]; pass 2 sums the partials in a
-// fixed order, so the result is deterministic.  Within a coordinate the
-// sums over the workers run in fp32 pairs (below) and only the coordinate's
-// totals in double: the GB300's fp64 rate is a small fraction of its fp32
-// rate, and per-worker fp64 arithmetic made the metrics fp64-bound.
+// fixed order, so the result is deterministic.  Within a quad the sums over
+// the workers run in fp32 pairs (below) and only the quad's totals in double:
+// the GB300's fp64 rate is a small fraction of its fp32 rate, and per-worker
+// fp64 arithmetic made the metrics fp64-bound.
 constexpr int kMetricsThreads = 256;
 constexpr int kMetricsMaxBlocks = 1024;
 
-// A running fp32 sum kept as the unevaluated pair s + c (Neumaier's
-// compensated summation): c gathers every addition's exact rounding error,
-// so the pair carries about twice fp32's precision.  The _rn intrinsics
-// keep the compiler from contracting or reordering the error terms.
+// The exact rounding error of a + b, given s = fl(a + b) (Knuth's TwoSum), of
+// two sums at once.
+__device__ __forceinline__ Pair sum_error(Pair a, Pair b, Pair s) {
+    const Pair bb = sub2(s, a);
+    return add2(sub2(a, sub2(s, bb)), sub2(b, bb));
+}
+
+// Two running fp32 sums, each kept as the unevaluated pair s + c: c gathers
+// every addition's exact rounding error, so the pair carries about twice
+// fp32's precision.  The packed instructions keep the compiler from
+// contracting or reordering the error terms.
 struct PairSum {
-    float s = 0.0f, c = 0.0f;
-    __device__ __forceinline__ void add(float v) {
-        const float t = __fadd_rn(s, v);
-        const float e = (fabsf(s) >= fabsf(v)) ? __fadd_rn(__fsub_rn(s, t), v) : __fadd_rn(__fsub_rn(v, t), s);
-        c = __fadd_rn(c, e);
+    Pair s = pack(0.0f), c = pack(0.0f);
+    __device__ __forceinline__ void add(Pair v) {
+        const Pair t = add2(s, v);
+        c = add2(c, sum_error(s, v, t));
         s = t;
     }
-    __device__ __forceinline__ double value() const { return static_cast<double>(s) + static_cast<double>(c); }
 };
-
-// The exact rounding error of a + b, given s = fl(a + b) (Knuth's TwoSum).
-__device__ __forceinline__ float sum_error(float a, float b, float s) {
-    const float bb = __fsub_rn(s, a);
-    return __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
-}
 
 __device__ __forceinline__ double block_sum(double v, double* red) {
     for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
@@ -122,52 +121,178 @@ __device__ __forceinline__ double block_sum(double v, double* red) {
     return s;  // valid in thread 0
 }
 
-template <int OBJ>
-__global__ void __launch_bounds__(kMetricsThreads)
+// 16 bytes of global memory into this thread's shared memory, asynchronously.
+__device__ __forceinline__ void copy_async(float4* dst, const float* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                     static_cast<uint32_t>(__cvta_generic_to_shared(dst))),
+                 "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void copies_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+// Waits until at most `Pending` of this thread's groups are outstanding.
+template <int Pending>
+__device__ __forceinline__ void copies_wait() {
+    asm volatile("cp.async.wait_group %0;" ::"n"(Pending) : "memory");
+}
+
+// sum_i (x_i - xbar)^2 of two coordinates: x_i - hi exactly as t + its
+// rounding error, less lo (dl); t^2 exactly as p + its fma remainder, and
+// 2 t dl + dl^2.
+struct SquareSum {
+    PairSum sq;
+    Pair lo = pack(0.0f);
+    __device__ __forceinline__ void add(Pair x, Pair minus_hi, Pair xbar_lo) {
+        const Pair t = add2(x, minus_hi);
+        const Pair dl = sub2(sum_error(x, minus_hi, t), xbar_lo);
+        const Pair p = mul2(t, t);
+        const Pair pe = fma2(t, t, mul2(p, pack(-1.0f)));
+        sq.add(p);
+        lo = add2(lo, fma2(dl, dl, fma2(add2(t, t), dl, pe)));
+    }
+};
+
+// Two values as the unevaluated fp32 pairs hi + lo.
+struct HiLo {
+    Pair hi, lo;
+};
+
+// (s + c) / n: the product with 1 / n as a pair of its own.
+__device__ __forceinline__ HiLo worker_mean(const PairSum& sum, Pair inv_hi, Pair inv_lo) {
+    const Pair t = add2(sum.s, sum.c);
+    const Pair e = sub2(sum.c, sub2(t, sum.s));
+    const Pair p = mul2(t, inv_hi);
+    const Pair r = fma2(e, inv_hi, fma2(t, inv_lo, fma2(t, inv_hi, mul2(p, pack(-1.0f)))));
+    const Pair hi = add2(p, r);
+    return HiLo{hi, sub2(r, sub2(hi, p))};
+}
+
+// Adds the squares (xbar - mubar)^2 of the two coordinates: the difference as
+// an fp32 pair, squared in double.
+__device__ __forceinline__ void add_squared_difference(const HiLo& x, const HiLo& m, double& total) {
+    const Pair minus_m = mul2(m.hi, pack(-1.0f));
+    const Pair t = add2(x.hi, minus_m);
+    const Pair el = add2(sum_error(x.hi, minus_m, t), sub2(x.lo, m.lo));
+    float t0, t1, l0, l1;
+    unpack(t, t0, t1);
+    unpack(el, l0, l1);
+    const double e0 = static_cast<double>(t0) + static_cast<double>(l0);
+    const double e1 = static_cast<double>(t1) + static_cast<double>(l1);
+    total += e0 * e0;
+    total += e1 * e1;
+}
+
+// Adds the four values of two pairs to a total kept in double: summed as fp32
+// pairs first, so a quad costs about 20 double-precision instructions and not
+// 80 (the GB300 does one of them per 64 of fp32; that bound the metrics of few
+// workers: 756 -> 232 us for 4 workers at d = 2.0e7).
+__device__ __forceinline__ void add_quad(const HiLo& a, const HiLo& b, double& total) {
+    const Pair t = add2(a.hi, b.hi);
+    const Pair e = add2(sum_error(a.hi, b.hi, t), add2(a.lo, b.lo));
+    float t0, t1, e0, e1;
+    unpack(t, t0, t1);
+    unpack(e, e0, e1);
+    const float s = __fadd_rn(t0, t1);
+    const float bb = __fsub_rn(s, t0);
+    const float err = __fadd_rn(__fsub_rn(t0, __fsub_rn(s, bb)), __fsub_rn(t1, bb));
+    total += static_cast<double>(s);
+    total += static_cast<double>(__fadd_rn(err, __fadd_rn(e0, e1)));
+}
+
+// Zeros the coordinates of a ragged last quad that lie beyond d: their values
+// are unspecified, and zeros add nothing.
+__device__ __forceinline__ float4 within(float4 v, int64_t c, int64_t d) {
+    if (c + 3 >= d) {
+        if (c + 1 >= d) v.y = 0.0f;
+        if (c + 2 >= d) v.z = 0.0f;
+        if (c + 3 >= d) v.w = 0.0f;
+    }
+    return v;
+}
+
+// STAGED: x crosses HBM once.  A thread keeps its quad of all n workers in a
+// shared-memory column ([i * blockDim] float4) between the two passes, filled
+// by asynchronous copies, its own only, so no barrier is needed: pass 1 waits
+// for a group of kMetricsGroup workers while the next kMetricsAhead groups
+// (and the stored centres, in a ring of their own) are in flight, and pass 2
+// starts the copy of the next quad's x_i as soon as it has used this one's.
+// 1,523 -> 1,210 us for 64 workers
+// at d = 9.2M, where one block of 4 warps fits an SM and its own latency is
+// what is left.  Without STAGED (more workers than the columns have room for,
+// or regenerated centres, which are bound by issue and want the resident
+// threads) pass 2 reads x again.
+constexpr int kMetricsBlock = 128;
+constexpr int kMetricsGroup = 4, kMetricsAhead = 3;
+constexpr int kMetricsRing = kMetricsGroup * (kMetricsAhead + 1);  // centres in flight or in use
+
+template <int OBJ, bool STAGED>
+__global__ void __launch_bounds__(STAGED ? kMetricsBlock : kMetricsThreads, STAGED ? 1 : 4)
 relay_metrics_kernel(const __grid_constant__ Objective obj, const __grid_constant__ PhiloxKey mu_key,
                      const __grid_constant__ ModelArgs a, int n, int64_t d, double* partials) {
+    allow_dependent_launch();
+    extern __shared__ float4 metrics_mem[];
     __shared__ double red[kMetricsThreads / 32];
+    const int threads = static_cast<int>(blockDim.x);
+    float4* const col = metrics_mem + threadIdx.x;  // [i * threads]: x_i
+    float4* const ring = col + n * threads;         // [(i % kMetricsRing) * threads]: stored mu_i
     double xi = 0.0, dist = 0.0;
-    const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
+    const int64_t stride = static_cast<int64_t>(gridDim.x) * threads;
     const double inv_n = 1.0 / n;
-    for (int64_t q = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; q < a.nquads; q += stride) {
-        PairSum xs[4], ms[4];
-        for (int i = 0; i < n; ++i) {
-            const float4 xv = *reinterpret_cast<const float4*>(a.x + i * a.ld_x + 4 * q);
-            const float4 mv = centre<OBJ>(obj, mu_key, a, i, q, nullptr, 0);
-            xs[0].add(xv.x); xs[1].add(xv.y); xs[2].add(xv.z); xs[3].add(xv.w);
-            ms[0].add(mv.x); ms[1].add(mv.y); ms[2].add(mv.z); ms[3].add(mv.w);
-        }
-        // xbar as the fp32 pair hi + lo
-        float hi[4], lo[4];
-        double xb[4];
-        for (int k = 0; k < 4; ++k) {
-            xb[k] = xs[k].value() * inv_n;
-            hi[k] = static_cast<float>(xb[k]);
-            lo[k] = static_cast<float>(xb[k] - static_cast<double>(hi[k]));
-        }
-        // sum_i (x_i - xbar)^2: x_i - hi exactly as t + its rounding error,
-        // less lo; t^2 exactly as p + its fma remainder
-        PairSum sq[4];
-        float sq_lo[4] = {0.f, 0.f, 0.f, 0.f};
-        for (int i = 0; i < n; ++i) {
-            const float4 xv = *reinterpret_cast<const float4*>(a.x + i * a.ld_x + 4 * q);
-            const float xk[4] = {xv.x, xv.y, xv.z, xv.w};
-            for (int k = 0; k < 4; ++k) {
-                const float t = __fsub_rn(xk[k], hi[k]);
-                const float dl = __fsub_rn(sum_error(xk[k], -hi[k], t), lo[k]);
-                const float p = __fmul_rn(t, t);
-                const float pe = __fmaf_rn(t, t, -p);
-                sq[k].add(p);
-                sq_lo[k] = __fadd_rn(sq_lo[k], __fmaf_rn(__fmul_rn(2.0f, t), dl, pe));
+    const float inv_f = static_cast<float>(inv_n);
+    const Pair inv_hi = pack(inv_f), inv_lo = pack(static_cast<float>(inv_n - static_cast<double>(inv_f)));
+    const int groups = (n + kMetricsGroup - 1) / kMetricsGroup;
+    int64_t q = static_cast<int64_t>(blockIdx.x) * threads + threadIdx.x;
+    if (STAGED) {
+        // the first quad's x, one commit group for all of it
+        if (q < a.nquads)
+            for (int i = 0; i < n; ++i) copy_async(col + i * threads, a.x + i * a.ld_x + 4 * q);
+        copies_commit();
+    }
+    for (; q < a.nquads; q += stride) {
+        PairSum xs[2], ms[2];
+        auto use = [&](float4 xv, float4 mv) {
+            xv = within(xv, 4 * q, d);
+            mv = within(mv, 4 * q, d);
+            xs[0].add(pack(xv.x, xv.y));
+            xs[1].add(pack(xv.z, xv.w));
+            ms[0].add(pack(mv.x, mv.y));
+            ms[1].add(pack(mv.z, mv.w));
+        };
+        if (STAGED) {
+            auto fetch = [&](int g) {  // group g's centres
+                if (OBJ == relaysum::kMuStored)
+                    for (int i = g * kMetricsGroup; i < min(n, (g + 1) * kMetricsGroup); ++i)
+                        copy_async(ring + (i % kMetricsRing) * threads, a.mu + i * a.ld_x + 4 * q);
+                copies_commit();
+            };
+            for (int g = 0; g < kMetricsAhead; ++g) fetch(g);
+            for (int g = 0; g < groups; ++g) {
+                fetch(g + kMetricsAhead);
+                copies_wait<kMetricsAhead>();  // group g (and x, committed before it) has arrived
+                for (int i = g * kMetricsGroup; i < min(n, (g + 1) * kMetricsGroup); ++i)
+                    use(col[i * threads],
+                        OBJ == relaysum::kMuStored ? ring[(i % kMetricsRing) * threads]
+                                                   : centre<OBJ>(obj, mu_key, a, i, q, nullptr, 0));
             }
+        } else {
+            for (int i = 0; i < n; ++i)
+                use(*reinterpret_cast<const float4*>(a.x + i * a.ld_x + 4 * q),
+                    centre<OBJ>(obj, mu_key, a, i, q, nullptr, 0));
         }
-        for (int k = 0; k < 4; ++k)
-            if (4 * q + k < d) {
-                xi += sq[k].value() + static_cast<double>(sq_lo[k]);
-                const double e = xb[k] - ms[k].value() * inv_n;
-                dist += e * e;
-            }
+        const HiLo xbar[2] = {worker_mean(xs[0], inv_hi, inv_lo), worker_mean(xs[1], inv_hi, inv_lo)};
+        const Pair minus_hi[2] = {mul2(xbar[0].hi, pack(-1.0f)), mul2(xbar[1].hi, pack(-1.0f))};
+        SquareSum sq[2];
+        const int64_t next = q + stride;
+        for (int i = 0; i < n; ++i) {
+            const float4 xv = within(
+                STAGED ? col[i * threads] : *reinterpret_cast<const float4*>(a.x + i * a.ld_x + 4 * q), 4 * q, d);
+            sq[0].add(pack(xv.x, xv.y), minus_hi[0], xbar[0].lo);
+            sq[1].add(pack(xv.z, xv.w), minus_hi[1], xbar[1].lo);
+            if (STAGED && next < a.nquads) copy_async(col + i * threads, a.x + i * a.ld_x + 4 * next);
+        }
+        if (STAGED) copies_commit();
+        add_quad(HiLo{sq[0].sq.s, add2(sq[0].sq.c, sq[0].lo)}, HiLo{sq[1].sq.s, add2(sq[1].sq.c, sq[1].lo)}, xi);
+        add_squared_difference(xbar[0], worker_mean(ms[0], inv_hi, inv_lo), dist);
+        add_squared_difference(xbar[1], worker_mean(ms[1], inv_hi, inv_lo), dist);
     }
     const double bxi = block_sum(xi, red);
     const double bdist = block_sum(dist, red);
@@ -179,6 +304,7 @@ relay_metrics_kernel(const __grid_constant__ Objective obj, const __grid_constan
 
 __global__ void relay_metrics_finish_kernel(const double* partials, int blocks, double scale_xi,
                                             double scale_dist, double* out) {
+    wait_for_prior_grid();
     __shared__ double red[kMetricsThreads / 32];
     double xi = 0.0, dist = 0.0;
     for (int b = threadIdx.x; b < blocks; b += blockDim.x) {
@@ -250,6 +376,43 @@ bool use_fused(const relay_handle* h) {
 bool is_small(const relay_handle* h) {
     return h->prog.n <= relaysum::kSmallN &&
            (h->obj.source == relaysum::kMuStored || h->obj.row_off[h->prog.n] <= relaysum::kSmallMixNnz);
+}
+
+// Shared memory a staged block takes, and the workers it has room for: 128
+// threads hold columns of up to 84 workers (200 KB).
+size_t metrics_smem(int n) { return static_cast<size_t>(n + kMetricsRing) * 16 * kMetricsBlock; }
+bool metrics_columns_fit(int n) { return metrics_smem(n) <= 200 * 1024; }
+
+template <int OBJ, bool STAGED>
+int launch_metrics_blocks(const relay_handle* h, const ModelArgs& a, int max_blocks, double* workspace, double* out,
+                          cudaStream_t stream) {
+    int dev = 0;
+    const int sms = device_sms(&dev);
+    if (sms <= 0) return RELAY_ECUDA;
+    const int n = h->prog.n;
+    const size_t smem = STAGED ? metrics_smem(n) : 0;
+    // The block size and count depend on the workers and coordinates alone, so
+    // stored and regenerated centres give the same bits.  Six blocks of 128 per
+    // SM at most: a whole number of waves when 1, 2, 3 or 6 are resident.
+    const int threads = metrics_columns_fit(n) ? kMetricsBlock : kMetricsThreads;
+    if (resident_ctas<relay_metrics_kernel<OBJ, STAGED>>(dev, threads, smem) <= 0) return RELAY_ECUDA;
+    const int blocks = std::min(max_blocks, (threads == kMetricsBlock ? 6 : 4) * sms);
+    const PhiloxKey mu_key = philox_key(static_cast<uint64_t>(h->obj.k0) | (static_cast<uint64_t>(h->obj.k1) << 32));
+    relay_metrics_kernel<OBJ, STAGED><<<blocks, threads, smem, stream>>>(h->obj, mu_key, a, n, h->d, workspace);
+    const int rc = launch_status();
+    if (rc != RELAY_OK) return rc;
+    const double denom = h->d > 0 ? static_cast<double>(h->d) : 1.0;
+    return launch_step_kernel(relay_metrics_finish_kernel, 1, kMetricsThreads, 0, stream, true,
+                              static_cast<const double*>(workspace), blocks, 1.0 / (n * denom), 1.0 / denom, out);
+}
+
+template <int OBJ>
+int launch_metrics(const relay_handle* h, const ModelArgs& a, int max_blocks, double* workspace, double* out,
+                   cudaStream_t stream) {
+    // regenerated centres are bound by issue, which wants the resident threads
+    if (OBJ == relaysum::kMuStored && metrics_columns_fit(h->prog.n))
+        return launch_metrics_blocks<OBJ, true>(h, a, max_blocks, workspace, out, stream);
+    return launch_metrics_blocks<OBJ, false>(h, a, max_blocks, workspace, out, stream);
 }
 
 // Rows of a message buffer: E, plus one received-sum row per wide node when
@@ -758,22 +921,10 @@ int relay_metrics(relay_handle* h, const float* x, double* workspace, double* ou
     a.ld_x = h->ld_x;
     a.nquads = h->nquads;
     a.q0 = static_cast<uint32_t>(h->c0 / 4);
-    const PhiloxKey mu_key = philox_key(static_cast<uint64_t>(h->obj.k0) | (static_cast<uint64_t>(h->obj.k1) << 32));
-    const int n = h->prog.n;
-    switch (h->obj.source) {
-        case relaysum::kMuStored:
-            relay_metrics_kernel<relaysum::kMuStored><<<blocks, kMetricsThreads, 0, stream>>>(
-                h->obj, mu_key, a, n, h->d, workspace);
-            break;
-        default:  // cached centres are regenerated per row here
-            relay_metrics_kernel<relaysum::kMuPerRow><<<blocks, kMetricsThreads, 0, stream>>>(
-                h->obj, mu_key, a, n, h->d, workspace);
-            break;
-    }
-    const double denom = h->d > 0 ? static_cast<double>(h->d) : 1.0;
-    relay_metrics_finish_kernel<<<1, kMetricsThreads, 0, stream>>>(workspace, blocks, 1.0 / (n * denom),
-                                                                   1.0 / denom, out);
-    return launch_status();
+    // cached centres are regenerated per row here
+    return h->obj.source == relaysum::kMuStored
+               ? launch_metrics<relaysum::kMuStored>(h, a, blocks, workspace, out, stream)
+               : launch_metrics<relaysum::kMuPerRow>(h, a, blocks, workspace, out, stream);
 }
 
 // ------------------------------------------- allocation-free metrics variant

@@ -79,3 +79,24 @@ def test_lr_correction_matches_oracle(shape, n):
     oracle.run(n, edges, x, mu, msg, c, 0.0, 0.0, 0, 1, 5000, 1)
     assert abs(alpha - x[:, 0].mean()) < 1e-5
     assert 0.0 < alpha < 1.0
+
+
+@pytest.mark.parametrize("n", [2, 84, 85])
+@pytest.mark.parametrize("d", [5, 515, 120_001])
+def test_metrics_at_the_edges_of_their_blocks(n, d):
+    """Blocks of 128 threads with shared-memory columns for up to 84 workers, of
+    256 without them above; ragged last quads whose columns beyond d hold NaN.
+    The bar is that of test_metrics_match_float64_definition."""
+    run = rs.RelayRun(n, d, wl.random_tree(n, 2), device="cuda:0")
+    run.init(0.3, 4, wl.identity_mix(n), 2.0, 5, 0.5)
+    for _ in range(2):
+        run.step(0.2, 4)
+    run.x[:, d:] = float("nan")
+    run.mu[:, d:] = float("nan")
+    m = run.metrics()[0].cpu().numpy()
+    assert np.allclose(m, _reference(run.x[:, :d].cpu().numpy(), run.mu[:, :d].cpu().numpy()), rtol=1e-9, atol=0)
+    regenerated = rs.RelayRun(n, d, wl.random_tree(n, 2), device="cuda:0", objective="generated")
+    regenerated.init(0.3, 4, wl.identity_mix(n), 2.0, 5, 0.5)
+    for _ in range(2):
+        regenerated.step(0.2, 4)
+    assert np.array_equal(regenerated.metrics()[0].cpu().numpy(), m)
