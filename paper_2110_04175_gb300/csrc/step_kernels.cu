@@ -481,95 +481,177 @@ relay_models_kernel(const __grid_constant__ Windows<NT> win, const __grid_consta
 // For short vectors the walk leaves the GPU idle (one thread per quad walks
 // all n workers in turn), so this form of the same step gives each
 // (worker, quad) pair its own thread.  A CTA owns qb consecutive quads of
-// every worker (threads worker-major: a worker's qb quads are contiguous).
-// Phase 1: each thread forms x_i^{t+1/2} and worker i's outgoing messages
-// with the walk's arithmetic (prefix + suffix at degree <= kRegDeg, the
-// total minus the reverse message above it), writes them out and leaves
-// them in shared memory.  Phase 2, after one barrier: each thread adds its
-// worker's incoming messages in the walk's order (Program::rb_in) and
-// writes the new model.  The results equal relay_models_kernel's bit for
-// bit, and every array is still read and written once.
+// every worker; qb consecutive threads share a worker, the workers in
+// ascending degree, so the lanes of a warp have (nearly) the same number of
+// messages.  Phase 1: each thread forms x_i^{t+1/2} and worker i's outgoing
+// messages with the walk's arithmetic (prefix + suffix at degree <= kRegDeg,
+// the total minus the reverse message above it), writes them out and leaves
+// them in shared memory, at the position where they arrive.  Phase 2, after
+// one barrier: each thread adds its worker's incoming messages, consecutive
+// rows in the walk's order, and writes the new model.  The results equal
+// relay_models_kernel's bit for bit, and every array is still read and
+// written once.
 
-// Degree D <= kRegDeg: outgoing message s = prefix(s) + suffix(s+1).
+// What a thread of the node-parallel and multi-step kernels is: one worker's
+// share of one quad at a time.
+struct NodeThread {
+    int i, deg;            // worker (deg 0 on the threads that fill up the last warp)
+    int pos_base;          // its first position
+    int in;                // float4 index of its first incoming message in a buffer; the next is qb further
+    uint32_t lost_bits;    // bit s: its message to neighbour s is lost (narrow nodes)
+};
+
+__device__ __forceinline__ NodeThread node_thread(const Program& prog, const ModelArgs& a, int slot, int qi, int qb) {
+    const bool live = slot < prog.n;
+    NodeThread t;
+    t.i = prog.by_degree[live ? slot : prog.n - 1];
+    t.deg = live ? prog.node[t.i].deg : 0;
+    t.pos_base = live ? prog.node[t.i].pos_base : 0;
+    t.in = t.pos_base * qb + qi;
+    t.lost_bits = 0;
+    if (a.has_lost && t.deg <= kRegDeg)
+        for (int s = 0; s < t.deg; ++s) t.lost_bits |= (a.lost(prog.pos_out[t.pos_base + s]) ? 1u : 0u) << s;
+    return t;
+}
+
+// Outgoing message s = prefix(s) + suffix(s + 1) with prefix(s) = xh + m_0 +
+// ... + m_{s-1}; the zeros of a lane's missing neighbours add nothing.
 template <int D>
-__device__ __forceinline__ void node_small(const Program& prog, const NodeRec& r, const ModelArgs& a,
-                                           int64_t q, float4 xh, float4* m_new, int qb) {
-    float4 m[D];
-#pragma unroll
-    for (int s = 0; s < D; ++s) m[s] = ld_stream(a.msg_in + prog.pos_in[r.pos_base + s] * a.ld_m + 4 * q);
-    float4 pre[D];
-    pre[0] = xh;
-#pragma unroll
-    for (int s = 1; s < D; ++s) pre[s] = add4(pre[s - 1], m[s - 1]);
+__device__ __forceinline__ void narrow_messages(const float4 (&m)[D], float4 xh, uint32_t lost_bits,
+                                                float4 (&o)[D]) {
+    float4 pre = xh;
     float4 suf[D];
     suf[D - 1] = m[D - 1];
 #pragma unroll
-    for (int s = D - 2; s >= 0; --s) suf[s] = add4(m[s], suf[s + 1]);
+    for (int s = D - 2; s >= 1; --s) suf[s] = add4(m[s], suf[s + 1]);
 #pragma unroll
     for (int s = 0; s < D; ++s) {
-        const int e = prog.pos_out[r.pos_base + s];
-        const float4 out = delivered(a, e, (s == D - 1) ? pre[s] : add4(pre[s], suf[s + 1]));
-        st_stream(a.msg_out + e * a.ld_m + 4 * q, out);
-        m_new[e * qb] = out;
+        o[s] = (s == D - 1) ? pre : add4(pre, suf[s + 1]);
+        if (s + 1 < D) pre = add4(pre, m[s]);
+    }
+    if (lost_bits) {
+#pragma unroll
+        for (int s = 0; s < D; ++s)
+            if ((lost_bits >> s) & 1u) o[s] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
 }
 
-// Degree D > kRegDeg: T = x^{t+1/2} + the incoming messages summed over
-// descending positions (with received sums: + the sum row S_i^{t-1}), then
-// message s = T - (incoming message s), as in visit_wide and at the wide
-// node's children.  The incoming messages wait in shared memory (rows of
-// worker i's own incoming edges).
-__device__ __noinline__ void node_wide(const Program& prog, const NodeRec& r, const ModelArgs& a, int i,
-                                       int64_t q, float4 xh, float4* m_new, float4* m_old, int qb) {
-    const int D = r.deg;
-    const int base = r.pos_base;
+// Phase 1 of a worker with at most D <= kRegDeg neighbours: its incoming rows
+// are requested before the noise arithmetic, which covers their latency (with
+// Adam after its update, whose registers they would spill: 40.7 against 40.2
+// us on the 16-worker chain at d = 272,474).  `sent[s]` is the float4 index where the message to neighbour s arrives.
+template <int D, int OPT>
+__device__ __forceinline__ float4 node_send(const Program& prog, const ModelArgs& a, const NodeThread& t, int64_t q,
+                                            float4 xv, float4 mv, const int (&sent)[kRegDeg], int qb, float4* m_new) {
+    constexpr int DN = D > 0 ? D : 1;
+    float4 m[DN];
+    auto request = [&]() {
+#pragma unroll
+        for (int s = 0; s < D; ++s) {
+            m[s] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (s < t.deg) m[s] = ld_stream(a.msg_in + prog.pos_in[t.pos_base + s] * a.ld_m + 4 * q);
+        }
+    };
+    if (OPT != 2) request();
+    const float4 z = minus_normal4(noise_words(noise_quad(a.q0 + static_cast<uint32_t>(q), a.key),
+                                               static_cast<uint32_t>(t.i), a.step, a.key));
+    const float4 xh = relayed_value<OPT>(a, t.i, q, xv, mv, z);
+    if (OPT == 2) request();
+    if (D > 0) {
+        float4 o[DN];
+        narrow_messages<DN>(m, xh, t.lost_bits, o);
+#pragma unroll
+        for (int s = 0; s < D; ++s)
+            if (s < t.deg) {
+                m_new[OPT == 2 ? prog.edge_pos[prog.pos_out[t.pos_base + s]] * qb + (t.in - t.pos_base * qb) : sent[s]] = o[s];
+                st_stream(a.msg_out + prog.pos_out[t.pos_base + s] * a.ld_m + 4 * q, o[s]);
+            }
+    }
+    return xh;
+}
+
+// Phase 1 in a warp with a worker of degree > kRegDeg: T = x^{t+1/2} + the
+// incoming messages summed over descending positions (with received sums: +
+// the sum row S_i^{t-1}), then message s = T - (incoming message s), as in
+// visit_wide and at the wide node's children.  The incoming messages wait in
+// shared memory (the worker's own rows of m_old).
+template <int OPT>
+__device__ __noinline__ float4 node_send_wide(const Program& prog, const ModelArgs& a, const NodeThread& t,
+                                              int64_t q, float4 xv, float4 mv, int qb, float4* m_new,
+                                              float4* m_old) {
+    const int qi = t.in - t.pos_base * qb;
+    const float4 z = minus_normal4(noise_words(noise_quad(a.q0 + static_cast<uint32_t>(q), a.key),
+                                               static_cast<uint32_t>(t.i), a.step, a.key));
+    const float4 xh = relayed_value<OPT>(a, t.i, q, xv, mv, z);
+    float4* const own = m_old + t.in;
+    const bool wide = t.deg > kRegDeg;
     float4 total = xh;
-    if (a.rsum) total = add4(xh, ld_stream(a.msg_in + rsum_row(prog, i) * a.ld_m + 4 * q));
-    for (int s = D - 1; s >= 0; --s) {
-        const int ein = prog.pos_in[base + s];
-        const float4 m = ld_stream(a.msg_in + ein * a.ld_m + 4 * q);
-        if (!a.rsum) total = add4(total, m);
-        m_old[ein * qb] = m;
+    if (wide && a.rsum) total = add4(xh, ld_stream(a.msg_in + rsum_row(prog, t.i) * a.ld_m + 4 * q));
+    for (int s = t.deg - 1; s >= 0; --s) {
+        const float4 m = ld_stream(a.msg_in + prog.pos_in[t.pos_base + s] * a.ld_m + 4 * q);
+        if (wide && !a.rsum) total = add4(total, m);
+        own[s * qb] = m;
     }
-    for (int s = 0; s < D; ++s) {
-        const int e = prog.pos_out[base + s];
-        const float4 out = delivered(a, e, sub4(total, m_old[prog.pos_in[base + s] * qb]));
-        st_stream(a.msg_out + e * a.ld_m + 4 * q, out);
-        m_new[e * qb] = out;
+    for (int s = 0; s < t.deg; ++s) {
+        float4 o;
+        if (wide) {
+            o = sub4(total, own[s * qb]);
+        } else {
+            o = xh;
+            for (int r = 0; r < s; ++r) o = add4(o, own[r * qb]);
+            if (s + 1 < t.deg) {
+                float4 suf = own[(t.deg - 1) * qb];
+                for (int r = t.deg - 2; r > s; --r) suf = add4(own[r * qb], suf);
+                o = add4(o, suf);
+            }
+        }
+        const int e = prog.pos_out[t.pos_base + s];
+        o = delivered(a, e, o);
+        st_stream(a.msg_out + e * a.ld_m + 4 * q, o);
+        m_new[prog.edge_pos[e] * qb + qi] = o;
     }
+    return xh;
 }
 
-// blockDim.x = qb * n <= 1024.  Dynamic shared memory: two [E][qb] float4
-// message buffers used by alternate blocks, plus one more for the incoming
-// messages of wide nodes when the tree has any.  With two buffers a block
-// needs one barrier: a warp already in the next block's phase 1 writes the
-// other buffer, and it can reach this buffer again only after every warp
-// has passed the next block's barrier, i.e. finished reading this one.
+// blockDim.x = qb * n rounded up to whole warps, at most kNodeThreads.
+// Dynamic shared memory: two [E][qb] float4 message buffers used by alternate
+// blocks, plus one more for the incoming messages of wide nodes when the tree
+// has any.  With two buffers a block needs one barrier: a warp already in the
+// next block's phase 1 writes the other buffer, and it can reach this buffer
+// again only after every warp has passed the next block's barrier, i.e.
+// finished reading this one.
+constexpr int kNodeThreads = 512;
+
 template <int OBJ, int OPT>
-__global__ void __launch_bounds__(1024)
+__global__ void __launch_bounds__(kNodeThreads, 2)
 relay_nodes_kernel(const __grid_constant__ Program prog, const __grid_constant__ ObjectiveArg<OBJ> obj,
-                   const __grid_constant__ PhiloxKey mu_key, const __grid_constant__ ModelArgs a, int qb) {
+                   const __grid_constant__ PhiloxKey mu_key, const __grid_constant__ ModelArgs a, int qb_log2) {
     extern __shared__ float4 node_mem[];
     __shared__ float s_scale[kMaxN];
     __shared__ float s_fill[kMaxN];
     // regenerated centres are formed per row (the walk's cached centres are
     // the same normals mixed in the same order)
     constexpr int kObj = (OBJ == relaysum::kMuStored) ? relaysum::kMuStored : relaysum::kMuPerRow;
-    const int i = static_cast<int>(threadIdx.x) / qb;
-    const int qi = static_cast<int>(threadIdx.x) - i * qb;
-    float4* const buf0 = node_mem + qi;                     // [e * qb]: m^t on edge e (even blocks)
-    float4* const buf1 = node_mem + prog.E * qb + qi;       // (odd blocks)
-    float4* const m_old = node_mem + 2 * prog.E * qb + qi;  // [e * qb]: m^{t-1} (wide nodes)
-    const NodeRec r = prog.node[i];
-    const float* const xrow = a.x + i * a.ld_x;
-    const float* const murow = (OBJ == relaysum::kMuStored) ? a.mu + i * a.ld_x : nullptr;
-    const int64_t nblk = (a.nquads + qb - 1) / qb;
-    const int64_t qstep = static_cast<int64_t>(gridDim.x) * qb;
+    const int qb = 1 << qb_log2;
+    const int tid = static_cast<int>(threadIdx.x);
+    const int slot = tid >> qb_log2, qi = tid & (qb - 1);
+    const bool live = slot < prog.n;
+    const NodeThread t = node_thread(prog, a, slot, qi, qb);
+    const int widest = __reduce_max_sync(0xffffffffu, t.deg);
+    int sent[kRegDeg];
+#pragma unroll
+    for (int s = 0; s < kRegDeg; ++s)
+        sent[s] = s < t.deg ? prog.edge_pos[prog.pos_out[t.pos_base + s]] * qb + qi : 0;
+    float4* const m_old = node_mem + 2 * prog.E * qb;
+    const float* const xrow = a.x + t.i * a.ld_x;
+    const float* const murow = (OBJ == relaysum::kMuStored) ? a.mu + t.i * a.ld_x : nullptr;
+    const int64_t nblk = (a.nquads + qb - 1) >> qb_log2;
+    const int64_t qstep = static_cast<int64_t>(gridDim.x) << qb_log2;
     // x (and a stored mu) of this thread's next block are loaded one block
     // early, so their latency overlaps the barrier and the rebuild
     float4 xn = make_float4(0.f, 0.f, 0.f, 0.f), mn = xn;
-    int64_t q = static_cast<int64_t>(blockIdx.x) * qb + qi;
-    if (q < a.nquads) {
+    int64_t q = (static_cast<int64_t>(blockIdx.x) << qb_log2) + qi;
+    if (live && q < a.nquads) {
         xn = *reinterpret_cast<const float4*>(xrow + 4 * q);
         if (OBJ == relaysum::kMuStored) mn = ld_stream(murow + 4 * q);
     }
@@ -580,26 +662,24 @@ relay_nodes_kernel(const __grid_constant__ Program prog, const __grid_constant__
     bool counted = false;
     int parity = 0;
     for (int64_t b = blockIdx.x; b < nblk; b += gridDim.x, q += qstep, parity ^= 1) {
-        float4* const m_new = parity ? buf1 : buf0;
-        const bool active = q < a.nquads;
+        float4* const m_new = node_mem + (parity ? prog.E * qb : 0);
+        const bool active = live && q < a.nquads;
         const float4 xv = xn, ms = mn;
-        if (q + qstep < a.nquads) {
+        if (live && q + qstep < a.nquads) {
             xn = *reinterpret_cast<const float4*>(xrow + 4 * (q + qstep));
             if (OBJ == relaysum::kMuStored) mn = ld_stream(murow + 4 * (q + qstep));
         }
         float4 xh = make_float4(0.f, 0.f, 0.f, 0.f);
         if (active) {
-            const float4 mv = (OBJ == relaysum::kMuStored) ? ms : centre<kObj>(obj, mu_key, a, i, q, nullptr, 0);
-            const float4 z = minus_normal4(noise_words(noise_quad(a.q0 + static_cast<uint32_t>(q), a.key),
-                                                       static_cast<uint32_t>(i), a.step, a.key));
-            xh = relayed_value<OPT>(a, i, q, xv, mv, z);
-            switch (r.deg) {
-                case 0: break;
-                case 1: node_small<1>(prog, r, a, q, xh, m_new, qb); break;
-                case 2: node_small<2>(prog, r, a, q, xh, m_new, qb); break;
-                case 3: node_small<3>(prog, r, a, q, xh, m_new, qb); break;
-                case 4: node_small<4>(prog, r, a, q, xh, m_new, qb); break;
-                default: node_wide(prog, r, a, i, q, xh, m_new, m_old, qb); break;
+            const float4 mv =
+                (OBJ == relaysum::kMuStored) ? ms : centre<kObj>(obj, mu_key, a, t.i, q, nullptr, 0);
+            switch (widest) {
+                case 0: xh = node_send<0, OPT>(prog, a, t, q, xv, mv, sent, qb, m_new); break;
+                case 1: xh = node_send<1, OPT>(prog, a, t, q, xv, mv, sent, qb, m_new); break;
+                case 2: xh = node_send<2, OPT>(prog, a, t, q, xv, mv, sent, qb, m_new); break;
+                case 3: xh = node_send<3, OPT>(prog, a, t, q, xv, mv, sent, qb, m_new); break;
+                case 4: xh = node_send<4, OPT>(prog, a, t, q, xv, mv, sent, qb, m_new); break;
+                default: xh = node_send_wide<OPT>(prog, a, t, q, xv, mv, qb, m_new, m_old); break;
             }
         }
         if (!counted) {
@@ -610,20 +690,24 @@ relay_nodes_kernel(const __grid_constant__ Program prog, const __grid_constant__
         __syncthreads();  // also publishes the factors
         if (active) {
             // the rebuild sum starts from fill_i x_i + x^{t+1/2}, as in the walk
+            const float4* const mine = m_new + t.in;
             float4 acc = xh;
-            if (s_fill[i] != 0.0f) acc = fma4(s_fill[i], xv, xh);
-            if (a.rsum && r.deg > kRegDeg) {  // and the wide node's received sum S_i^t, in the same order
+            if (s_fill[t.i] != 0.0f) acc = fma4(s_fill[t.i], xv, xh);
+            if (t.deg <= kRegDeg) {
+#pragma unroll
+                for (int s = 0; s < kRegDeg; ++s)
+                    if (s < t.deg) acc = add4(acc, mine[s * qb]);
+            } else if (a.rsum) {  // and the wide node's received sum S_i^t, in the same order
                 float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
-                for (int k = 0; k < r.deg; ++k) {
-                    const float4 m = m_new[prog.pos_in[r.pos_base + k] * qb];
-                    acc = add4(acc, m);
-                    sum = add4(sum, m);
+                for (int s = 0; s < t.deg; ++s) {
+                    acc = add4(acc, mine[s * qb]);
+                    sum = add4(sum, mine[s * qb]);
                 }
-                st_stream(a.msg_out + rsum_row(prog, i) * a.ld_m + 4 * q, sum);
+                st_stream(a.msg_out + rsum_row(prog, t.i) * a.ld_m + 4 * q, sum);
             } else {
-                for (int k = 0; k < r.deg; ++k) acc = add4(acc, m_new[prog.pos_in[r.pos_base + k] * qb]);
+                for (int s = 0; s < t.deg; ++s) acc = add4(acc, mine[s * qb]);
             }
-            st_stream(a.x + i * a.ld_x + 4 * q, scale4(acc, s_scale[i]));
+            st_stream(a.x + t.i * a.ld_x + 4 * q, scale4(acc, s_scale[t.i]));
         }
     }
 }
@@ -644,15 +728,6 @@ relay_nodes_kernel(const __grid_constant__ Program prog, const __grid_constant__
 // places in the code, one per number of neighbours.
 __device__ __forceinline__ void cta_barrier() { asm volatile("bar.sync 1, %0;" ::"r"(blockDim.x) : "memory"); }
 
-// What a thread of relay_fused_steps_kernel is: one worker's share of one
-// quad at a time.
-struct FusedThread {
-    int i, deg;            // worker (deg 0 on the threads that fill up the last warp)
-    int pos_base;          // its first position
-    int in;                // float4 index of its first incoming message in a buffer; the next is qb further
-    uint32_t lost_bits;    // bit s: its message to neighbour s is lost (narrow nodes)
-};
-
 // One launch's k steps of one quad for a warp whose workers all have at most
 // D neighbours (D <= kRegDeg; a lane with fewer skips the missing ones).
 // The messages that arrived at the step before are registers m: they are read
@@ -663,7 +738,7 @@ struct FusedThread {
 // nothing here, is drawn between the loads of the new messages and their use.
 template <int D, int OPT, bool PLAIN>
 __device__ __forceinline__ void fused_steps(const Program& prog, const ModelArgs& a, const FusedSteps& fs,
-                                            const FusedThread& t, const float2* factors, float4* buf, int buf_len,
+                                            const NodeThread& t, const float2* factors, float4* buf, int buf_len,
                                             int qb, int& parity, bool active, int64_t q, float4& xv, float4 mv,
                                             float4& m1, float4& m2) {
     constexpr int DN = D > 0 ? D : 1;
@@ -697,24 +772,8 @@ __device__ __forceinline__ void fused_steps(const Program& prog, const ModelArgs
         float4* const cur = buf + (parity ? buf_len : 0);
         parity ^= 1;
         if (D > 0) {
-            // outgoing message s = prefix(s) + suffix(s + 1), as node_small
             float4 o[DN];
-            float4 pre = xh;
-            float4 suf[DN];
-            suf[DN - 1] = m[DN - 1];
-#pragma unroll
-            for (int s = D - 2; s >= 1; --s) suf[s] = add4(m[s], suf[s + 1]);
-#pragma unroll
-            for (int s = 0; s < D; ++s) {
-                // the zeros of a lane's missing neighbours add nothing
-                o[s] = (s == D - 1) ? pre : add4(pre, suf[s + 1]);
-                if (s + 1 < D) pre = add4(pre, m[s]);
-            }
-            if (t.lost_bits) {
-#pragma unroll
-                for (int s = 0; s < D; ++s)
-                    if ((t.lost_bits >> s) & 1u) o[s] = zero;
-            }
+            narrow_messages<DN>(m, xh, t.lost_bits, o);
 #pragma unroll
             for (int s = 0; s < D; ++s)
                 if (s < t.deg) cur[out[s]] = o[s];
@@ -744,10 +803,10 @@ __device__ __forceinline__ void fused_steps(const Program& prog, const ModelArgs
 // The same for a warp with a worker of degree > kRegDeg (a star's hub): the
 // messages that arrived at the step before stay in shared memory, in the
 // worker's own rows of the other buffer, and the outgoing ones are formed as
-// node_small and node_wide form them.
+// node_send_wide forms them.
 template <int OPT>
 __device__ __noinline__ void fused_steps_wide(const Program& prog, const ModelArgs& a, const FusedSteps& fs,
-                                              const FusedThread& t, const float2* factors, float4* buf, int buf_len,
+                                              const NodeThread& t, const float2* factors, float4* buf, int buf_len,
                                               int qb, int& parity, bool active, int64_t q, float4& xv, float4 mv,
                                               float4& m1, float4& m2) {
     const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -847,14 +906,7 @@ relay_fused_steps_kernel(const __grid_constant__ Program prog, const __grid_cons
     const int slot = tid >> fs.qb_log2;
     const int qi = tid & (qb - 1);
     const bool live = slot < n;
-    FusedThread t;
-    t.i = prog.by_degree[live ? slot : n - 1];
-    t.deg = live ? prog.node[t.i].deg : 0;
-    t.pos_base = live ? prog.node[t.i].pos_base : 0;
-    t.in = t.pos_base * qb + qi;
-    t.lost_bits = 0;
-    if (a.has_lost && t.deg <= kRegDeg)
-        for (int s = 0; s < t.deg; ++s) t.lost_bits |= (a.lost(prog.pos_out[t.pos_base + s]) ? 1u : 0u) << s;
+    const NodeThread t = node_thread(prog, a, slot, qi, qb);
     const int widest = __reduce_max_sync(0xffffffffu, t.deg);
     const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
     const int64_t nblk = (a.nquads + qb - 1) >> fs.qb_log2;
@@ -951,30 +1003,32 @@ int launch_models(const relay_handle* const* hs, const ModelArgs* as, cudaStream
                               after_counts, win, objective_of<OBJ>(hs[0]), mu_key);
 }
 
-// Quads per CTA of the node-parallel kernel, threads = qb * n <= 1024: a
-// whole warp per worker up to n = 16 (every per-worker table read is then
-// warp-uniform), half a warp up to 64, then 8 and 4 quads.
-int nodes_qb(int n) { return n <= 16 ? 32 : n <= 64 ? 16 : n <= 128 ? 8 : 4; }
+// Quads per CTA of the node-parallel kernel, as a power of two: as many as
+// fill kNodeThreads, at most a warp's worth (a whole warp per worker up to 16
+// workers).
+int nodes_qb_log2(int n) {
+    int l = 5;
+    while (l > 0 && (n << l) > kNodeThreads) --l;
+    return l;
+}
 
 template <int OBJ, int OPT>
 int launch_nodes(const relay_handle* h, const ModelArgs& a, cudaStream_t stream, bool after_counts) {
     int dev = 0;
     const int sms = device_sms(&dev);
     if (sms <= 0) return RELAY_ECUDA;
-    const int qb = nodes_qb(h->prog.n);
-    const int threads = qb * h->prog.n;
-    bool wide = false;
-    for (int i = 0; i < h->prog.n; ++i) wide = wide || h->prog.node[i].deg > kRegDeg;
-    const size_t smem = static_cast<size_t>(wide ? 3 : 2) * h->prog.E * qb * 16;
+    const int qb_log2 = nodes_qb_log2(h->prog.n);
+    const int threads = ((h->prog.n << qb_log2) + 31) / 32 * 32;
+    const size_t smem = (static_cast<size_t>(has_wide(h) ? 3 : 2) * h->prog.E << qb_log2) * 16;
     if (smem > static_cast<size_t>(kMaxSmem)) return RELAY_EUNSUPPORTED;
     const int per_sm = resident_ctas<relay_nodes_kernel<OBJ, OPT>>(dev, threads, smem);
     if (per_sm <= 0) return RELAY_ECUDA;
-    const int64_t want = (a.nquads + qb - 1) / qb;
+    const int64_t want = (a.nquads + (int64_t(1) << qb_log2) - 1) >> qb_log2;
     const int64_t cap = static_cast<int64_t>(sms) * per_sm;
     const int grid = static_cast<int>(want < cap ? want : cap);
     const PhiloxKey mu_key = philox_key(static_cast<uint64_t>(h->obj.k0) | (static_cast<uint64_t>(h->obj.k1) << 32));
     return launch_step_kernel(relay_nodes_kernel<OBJ, OPT>, grid, threads, smem, stream, after_counts,
-                              program_of(h), objective_of<OBJ>(h), mu_key, a, qb);
+                              program_of(h), objective_of<OBJ>(h), mu_key, a, qb_log2);
 }
 
 // Whether the walk over narrow trees with stored centres runs 7 CTAs per SM
