@@ -861,7 +861,7 @@ __device__ __noinline__ void fused_steps_wide(const Program& prog, const ModelAr
     }
 }
 
-// blockDim.x = qb * n rounded up to whole warps, at most kFusedThreads; qb
+// blockDim.x = qb * n rounded up to whole warps, at most THREADS; qb
 // consecutive threads share a worker, the workers in ascending degree, so
 // that the workers of one warp have (nearly) the same number of neighbours
 // and no lane waits for another's longer code path.  Dynamic shared memory:
@@ -870,10 +870,19 @@ __device__ __noinline__ void fused_steps_wide(const Program& prog, const ModelAr
 // factors (scale, fill) of every worker and counter round, [rounds][n]
 // float2.  The counters, hence the factors, are the same for every quad: the
 // CTA advances them once, before its first quads.
-constexpr int kFusedThreads = 512;
+//
+// THREADS: up to 32 workers take CTAs of at most 256 threads, three per SM
+// with 80 registers, where the barrier holds fewer warps and nothing spills
+// in the loop: against 512 threads, two per SM with 64 registers, 510 -> 491
+// us (16-worker binary tree, d = 272,474, 64 steps), 30.7 -> 28.7 us (8-worker
+// chain, d = 4,096), 806 -> 785 us with Adam.  More workers keep 512, since
+// half of it would leave rows of 4 quads: 362 against 351 us on the 64-worker
+// chain at d = 30,001.
+constexpr int kFusedFewWorkers = 32;
+constexpr int fused_threads(int n) { return n <= kFusedFewWorkers ? 256 : 512; }
 
-template <int OBJ, int OPT, bool PLAIN>
-__global__ void __launch_bounds__(kFusedThreads, 2)
+template <int OBJ, int OPT, bool PLAIN, int THREADS>
+__global__ void __launch_bounds__(THREADS, THREADS == 256 ? 3 : 2)
 relay_fused_steps_kernel(const __grid_constant__ Program prog, const __grid_constant__ ObjectiveArg<OBJ> obj,
                          const __grid_constant__ PhiloxKey mu_key, const __grid_constant__ ModelArgs a,
                          const __grid_constant__ FusedSteps fs) {
@@ -1081,17 +1090,17 @@ int launch_models_obj(const relay_handle* h, const ModelArgs& a, bool nodes, cud
 }
 
 // Quads per CTA of relay_fused_steps_kernel (as a power of two): as many as
-// fill kFusedThreads, at most a warp's worth, halved while that leaves fewer
+// fill its threads, at most a warp's worth, halved while that leaves fewer
 // CTAs than SMs (short vectors then still spread over the whole GPU) and the
 // CTA keeps a full warp.
 int fused_qb_log2(int n, int64_t nquads, int sms) {
     int l = 5;
-    while (l > 0 && (n << l) > kFusedThreads) --l;
+    while (l > 0 && (n << l) > fused_threads(n)) --l;
     while (l > 0 && (n << (l - 1)) >= 32 && (nquads + (int64_t(1) << l) - 1) >> l < sms) --l;
     return l;
 }
 
-template <int OBJ, int OPT, bool PLAIN>
+template <int OBJ, int OPT, bool PLAIN, int THREADS>
 int launch_fused(const relay_handle* h, const ModelArgs& a, FusedSteps& fs, cudaStream_t stream) {
     int dev = 0;
     const int sms = device_sms(&dev);
@@ -1101,24 +1110,30 @@ int launch_fused(const relay_handle* h, const ModelArgs& a, FusedSteps& fs, cuda
     const int threads = ((n << fs.qb_log2) + 31) / 32 * 32;
     const size_t smem = (static_cast<size_t>(2) * h->prog.E << fs.qb_log2) * 16 + static_cast<size_t>(fs.rounds) * n * 8;
     if (smem > static_cast<size_t>(kMaxSmem)) return RELAY_EUNSUPPORTED;
-    const int per_sm = resident_ctas<relay_fused_steps_kernel<OBJ, OPT, PLAIN>>(dev, threads, smem);
+    const int per_sm = resident_ctas<relay_fused_steps_kernel<OBJ, OPT, PLAIN, THREADS>>(dev, threads, smem);
     if (per_sm <= 0) return RELAY_ECUDA;
     const int64_t want = (a.nquads + (int64_t(1) << fs.qb_log2) - 1) >> fs.qb_log2;
     const int64_t cap = static_cast<int64_t>(sms) * per_sm;
     const int grid = static_cast<int>(want < cap ? want : cap);
     const PhiloxKey mu_key = philox_key(static_cast<uint64_t>(h->obj.k0) | (static_cast<uint64_t>(h->obj.k1) << 32));
-    relay_fused_steps_kernel<OBJ, OPT, PLAIN><<<grid, threads, smem, stream>>>(program_of(h), objective_of<OBJ>(h), mu_key, a, fs);
+    relay_fused_steps_kernel<OBJ, OPT, PLAIN, THREADS><<<grid, threads, smem, stream>>>(program_of(h), objective_of<OBJ>(h), mu_key, a, fs);
     return launch_status();
+}
+
+template <int OBJ, int OPT, bool PLAIN>
+int launch_fused_threads(const relay_handle* h, const ModelArgs& a, FusedSteps& fs, cudaStream_t stream) {
+    return fused_threads(h->prog.n) == 256 ? launch_fused<OBJ, OPT, PLAIN, 256>(h, a, fs, stream)
+                                           : launch_fused<OBJ, OPT, PLAIN, 512>(h, a, fs, stream);
 }
 
 template <int OPT>
 int launch_fused_obj(const relay_handle* h, const ModelArgs& a, FusedSteps& fs, cudaStream_t stream) {
     const bool plain = h->algo == RELAY_ALGO_RELAYSGD;
     if (h->obj.source == relaysum::kMuStored)
-        return plain ? launch_fused<relaysum::kMuStored, OPT, true>(h, a, fs, stream)
-                     : launch_fused<relaysum::kMuStored, OPT, false>(h, a, fs, stream);
-    return plain ? launch_fused<relaysum::kMuPerRow, OPT, true>(h, a, fs, stream)
-                 : launch_fused<relaysum::kMuPerRow, OPT, false>(h, a, fs, stream);
+        return plain ? launch_fused_threads<relaysum::kMuStored, OPT, true>(h, a, fs, stream)
+                     : launch_fused_threads<relaysum::kMuStored, OPT, false>(h, a, fs, stream);
+    return plain ? launch_fused_threads<relaysum::kMuPerRow, OPT, true>(h, a, fs, stream)
+                 : launch_fused_threads<relaysum::kMuPerRow, OPT, false>(h, a, fs, stream);
 }
 
 // Window k of a counter launch: handle h's program, lost mask and arrays.
