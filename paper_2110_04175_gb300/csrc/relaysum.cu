@@ -87,6 +87,7 @@ __global__ void relay_fill_mu_kernel(float* mu, const float* mix, int n, int K, 
 // the GB300's fp64 rate is a small fraction of its fp32 rate, and per-worker
 // fp64 arithmetic made the metrics fp64-bound.
 constexpr int kMetricsThreads = 256;
+constexpr int kMetricsResident = 4;  // blocks per SM: one wave of equal shares
 constexpr int kMetricsMaxBlocks = 1024;
 
 // The exact rounding error of a + b, given s = fl(a + b) (Knuth's TwoSum), of
@@ -119,20 +120,6 @@ __device__ __forceinline__ double block_sum(double v, double* red) {
     if (threadIdx.x == 0)
         for (int w = 0; w < static_cast<int>(blockDim.x >> 5); ++w) s += red[w];
     return s;  // valid in thread 0
-}
-
-// 16 bytes of global memory into this thread's shared memory, asynchronously.
-__device__ __forceinline__ void copy_async(float4* dst, const float* src) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
-                     static_cast<uint32_t>(__cvta_generic_to_shared(dst))),
-                 "l"(src)
-                 : "memory");
-}
-__device__ __forceinline__ void copies_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-// Waits until at most `Pending` of this thread's groups are outstanding.
-template <int Pending>
-__device__ __forceinline__ void copies_wait() {
-    asm volatile("cp.async.wait_group %0;" ::"n"(Pending) : "memory");
 }
 
 // sum_i (x_i - xbar)^2 of two coordinates: x_i - hi exactly as t + its
@@ -184,7 +171,7 @@ __device__ __forceinline__ void add_squared_difference(const HiLo& x, const HiLo
 // Adds the four values of two pairs to a total kept in double: summed as fp32
 // pairs first, so a quad costs about 20 double-precision instructions and not
 // 80 (the GB300 does one of them per 64 of fp32; that bound the metrics of few
-// workers: 756 -> 232 us for 4 workers at d = 2.0e7).
+// workers: 756 -> 221 us for 4 workers at d = 2.0e7).
 __device__ __forceinline__ void add_quad(const HiLo& a, const HiLo& b, double& total) {
     const Pair t = add2(a.hi, b.hi);
     const Pair e = add2(sum_error(a.hi, b.hi, t), add2(a.lo, b.lo));
@@ -209,87 +196,39 @@ __device__ __forceinline__ float4 within(float4 v, int64_t c, int64_t d) {
     return v;
 }
 
-// STAGED: x crosses HBM once.  A thread keeps its quad of all n workers in a
-// shared-memory column ([i * blockDim] float4) between the two passes, filled
-// by asynchronous copies, its own only, so no barrier is needed: pass 1 waits
-// for a group of kMetricsGroup workers while the next kMetricsAhead groups
-// (and the stored centres, in a ring of their own) are in flight, and pass 2
-// starts the copy of the next quad's x_i as soon as it has used this one's.
-// 1,523 -> 1,210 us for 64 workers
-// at d = 9.2M, where one block of 4 warps fits an SM and its own latency is
-// what is left.  Without STAGED (more workers than the columns have room for,
-// or regenerated centres, which are bound by issue and want the resident
-// threads) pass 2 reads x again.
-constexpr int kMetricsBlock = 128;
-constexpr int kMetricsGroup = 4, kMetricsAhead = 3;
-constexpr int kMetricsRing = kMetricsGroup * (kMetricsAhead + 1);  // centres in flight or in use
-
-template <int OBJ, bool STAGED>
-__global__ void __launch_bounds__(STAGED ? kMetricsBlock : kMetricsThreads, STAGED ? 1 : 4)
+// Bound by issue and the second read of x (from L2 in part): 1,156 us for 64
+// workers at d = 9.2M, 1,523 with scalar arithmetic and the means in double.
+// Keeping a quad's x_i in shared memory between the passes, filled by
+// asynchronous copies, left one block of 4 warps per SM and 1,214 us.
+template <int OBJ>
+__global__ void __launch_bounds__(kMetricsThreads, kMetricsResident)
 relay_metrics_kernel(const __grid_constant__ Objective obj, const __grid_constant__ PhiloxKey mu_key,
                      const __grid_constant__ ModelArgs a, int n, int64_t d, double* partials) {
     allow_dependent_launch();
-    extern __shared__ float4 metrics_mem[];
     __shared__ double red[kMetricsThreads / 32];
-    const int threads = static_cast<int>(blockDim.x);
-    float4* const col = metrics_mem + threadIdx.x;  // [i * threads]: x_i
-    float4* const ring = col + n * threads;         // [(i % kMetricsRing) * threads]: stored mu_i
     double xi = 0.0, dist = 0.0;
-    const int64_t stride = static_cast<int64_t>(gridDim.x) * threads;
+    const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
     const double inv_n = 1.0 / n;
     const float inv_f = static_cast<float>(inv_n);
     const Pair inv_hi = pack(inv_f), inv_lo = pack(static_cast<float>(inv_n - static_cast<double>(inv_f)));
-    const int groups = (n + kMetricsGroup - 1) / kMetricsGroup;
-    int64_t q = static_cast<int64_t>(blockIdx.x) * threads + threadIdx.x;
-    if (STAGED) {
-        // the first quad's x, one commit group for all of it
-        if (q < a.nquads)
-            for (int i = 0; i < n; ++i) copy_async(col + i * threads, a.x + i * a.ld_x + 4 * q);
-        copies_commit();
-    }
-    for (; q < a.nquads; q += stride) {
+    for (int64_t q = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; q < a.nquads; q += stride) {
         PairSum xs[2], ms[2];
-        auto use = [&](float4 xv, float4 mv) {
-            xv = within(xv, 4 * q, d);
-            mv = within(mv, 4 * q, d);
+        for (int i = 0; i < n; ++i) {
+            const float4 xv = within(*reinterpret_cast<const float4*>(a.x + i * a.ld_x + 4 * q), 4 * q, d);
+            const float4 mv = within(centre<OBJ>(obj, mu_key, a, i, q, nullptr, 0), 4 * q, d);
             xs[0].add(pack(xv.x, xv.y));
             xs[1].add(pack(xv.z, xv.w));
             ms[0].add(pack(mv.x, mv.y));
             ms[1].add(pack(mv.z, mv.w));
-        };
-        if (STAGED) {
-            auto fetch = [&](int g) {  // group g's centres
-                if (OBJ == relaysum::kMuStored)
-                    for (int i = g * kMetricsGroup; i < min(n, (g + 1) * kMetricsGroup); ++i)
-                        copy_async(ring + (i % kMetricsRing) * threads, a.mu + i * a.ld_x + 4 * q);
-                copies_commit();
-            };
-            for (int g = 0; g < kMetricsAhead; ++g) fetch(g);
-            for (int g = 0; g < groups; ++g) {
-                fetch(g + kMetricsAhead);
-                copies_wait<kMetricsAhead>();  // group g (and x, committed before it) has arrived
-                for (int i = g * kMetricsGroup; i < min(n, (g + 1) * kMetricsGroup); ++i)
-                    use(col[i * threads],
-                        OBJ == relaysum::kMuStored ? ring[(i % kMetricsRing) * threads]
-                                                   : centre<OBJ>(obj, mu_key, a, i, q, nullptr, 0));
-            }
-        } else {
-            for (int i = 0; i < n; ++i)
-                use(*reinterpret_cast<const float4*>(a.x + i * a.ld_x + 4 * q),
-                    centre<OBJ>(obj, mu_key, a, i, q, nullptr, 0));
         }
         const HiLo xbar[2] = {worker_mean(xs[0], inv_hi, inv_lo), worker_mean(xs[1], inv_hi, inv_lo)};
         const Pair minus_hi[2] = {mul2(xbar[0].hi, pack(-1.0f)), mul2(xbar[1].hi, pack(-1.0f))};
         SquareSum sq[2];
-        const int64_t next = q + stride;
         for (int i = 0; i < n; ++i) {
-            const float4 xv = within(
-                STAGED ? col[i * threads] : *reinterpret_cast<const float4*>(a.x + i * a.ld_x + 4 * q), 4 * q, d);
+            const float4 xv = within(*reinterpret_cast<const float4*>(a.x + i * a.ld_x + 4 * q), 4 * q, d);
             sq[0].add(pack(xv.x, xv.y), minus_hi[0], xbar[0].lo);
             sq[1].add(pack(xv.z, xv.w), minus_hi[1], xbar[1].lo);
-            if (STAGED && next < a.nquads) copy_async(col + i * threads, a.x + i * a.ld_x + 4 * next);
         }
-        if (STAGED) copies_commit();
         add_quad(HiLo{sq[0].sq.s, add2(sq[0].sq.c, sq[0].lo)}, HiLo{sq[1].sq.s, add2(sq[1].sq.c, sq[1].lo)}, xi);
         add_squared_difference(xbar[0], worker_mean(ms[0], inv_hi, inv_lo), dist);
         add_squared_difference(xbar[1], worker_mean(ms[1], inv_hi, inv_lo), dist);
@@ -378,41 +317,21 @@ bool is_small(const relay_handle* h) {
            (h->obj.source == relaysum::kMuStored || h->obj.row_off[h->prog.n] <= relaysum::kSmallMixNnz);
 }
 
-// Shared memory a staged block takes, and the workers it has room for: 128
-// threads hold columns of up to 84 workers (200 KB).
-size_t metrics_smem(int n) { return static_cast<size_t>(n + kMetricsRing) * 16 * kMetricsBlock; }
-bool metrics_columns_fit(int n) { return metrics_smem(n) <= 200 * 1024; }
-
-template <int OBJ, bool STAGED>
-int launch_metrics_blocks(const relay_handle* h, const ModelArgs& a, int max_blocks, double* workspace, double* out,
-                          cudaStream_t stream) {
+template <int OBJ>
+int launch_metrics(const relay_handle* h, const ModelArgs& a, int max_blocks, double* workspace, double* out,
+                   cudaStream_t stream) {
     int dev = 0;
     const int sms = device_sms(&dev);
     if (sms <= 0) return RELAY_ECUDA;
     const int n = h->prog.n;
-    const size_t smem = STAGED ? metrics_smem(n) : 0;
-    // The block size and count depend on the workers and coordinates alone, so
-    // stored and regenerated centres give the same bits.  Six blocks of 128 per
-    // SM at most: a whole number of waves when 1, 2, 3 or 6 are resident.
-    const int threads = metrics_columns_fit(n) ? kMetricsBlock : kMetricsThreads;
-    if (resident_ctas<relay_metrics_kernel<OBJ, STAGED>>(dev, threads, smem) <= 0) return RELAY_ECUDA;
-    const int blocks = std::min(max_blocks, (threads == kMetricsBlock ? 6 : 4) * sms);
+    const int blocks = std::min(max_blocks, kMetricsResident * sms);
     const PhiloxKey mu_key = philox_key(static_cast<uint64_t>(h->obj.k0) | (static_cast<uint64_t>(h->obj.k1) << 32));
-    relay_metrics_kernel<OBJ, STAGED><<<blocks, threads, smem, stream>>>(h->obj, mu_key, a, n, h->d, workspace);
+    relay_metrics_kernel<OBJ><<<blocks, kMetricsThreads, 0, stream>>>(h->obj, mu_key, a, n, h->d, workspace);
     const int rc = launch_status();
     if (rc != RELAY_OK) return rc;
     const double denom = h->d > 0 ? static_cast<double>(h->d) : 1.0;
     return launch_step_kernel(relay_metrics_finish_kernel, 1, kMetricsThreads, 0, stream, true,
                               static_cast<const double*>(workspace), blocks, 1.0 / (n * denom), 1.0 / denom, out);
-}
-
-template <int OBJ>
-int launch_metrics(const relay_handle* h, const ModelArgs& a, int max_blocks, double* workspace, double* out,
-                   cudaStream_t stream) {
-    // regenerated centres are bound by issue, which wants the resident threads
-    if (OBJ == relaysum::kMuStored && metrics_columns_fit(h->prog.n))
-        return launch_metrics_blocks<OBJ, true>(h, a, max_blocks, workspace, out, stream);
-    return launch_metrics_blocks<OBJ, false>(h, a, max_blocks, workspace, out, stream);
 }
 
 // Rows of a message buffer: E, plus one received-sum row per wide node when

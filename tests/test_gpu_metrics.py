@@ -81,11 +81,10 @@ def test_lr_correction_matches_oracle(shape, n):
     assert 0.0 < alpha < 1.0
 
 
-@pytest.mark.parametrize("n", [2, 84, 85])
+@pytest.mark.parametrize("n", [1, 2, 85])
 @pytest.mark.parametrize("d", [5, 515, 120_001])
 def test_metrics_at_the_edges_of_their_blocks(n, d):
-    """Blocks of 128 threads with shared-memory columns for up to 84 workers, of
-    256 without them above; ragged last quads whose columns beyond d hold NaN.
+    """One block and many, ragged last quads whose columns beyond d hold NaN.
     The bar is that of test_metrics_match_float64_definition."""
     run = rs.RelayRun(n, d, wl.random_tree(n, 2), device="cuda:0")
     run.init(0.3, 4, wl.identity_mix(n), 2.0, 5, 0.5)
