@@ -732,6 +732,10 @@ relay_nodes_kernel(const __grid_constant__ Program prog, const __grid_constant__
 // places in the code, one per number of neighbours.
 __device__ __forceinline__ void cta_barrier() { asm volatile("bar.sync 1, %0;" ::"r"(blockDim.x) : "memory"); }
 
+// Both message buffers are written before the launch ends (the one that step
+// t0 reads holds the messages of one of the last two steps), so they are read
+// with ordinary loads, not non-coherent ones.
+//
 // One launch's k steps of one quad for a warp whose workers all have at most
 // D neighbours (D <= kRegDeg; a lane with fewer skips the missing ones).
 // The messages that arrived at the step before are registers m: they are read
@@ -756,7 +760,7 @@ __device__ __forceinline__ void fused_steps(const Program& prog, const ModelArgs
         if (s < t.deg) {
             // where the message to neighbour s arrives
             out[s] = prog.edge_pos[prog.pos_out[t.pos_base + s]] * qb + (t.in - t.pos_base * qb);
-            if (active) m[s] = ld_stream(a.msg_in + prog.pos_in[t.pos_base + s] * a.ld_m + 4 * q);
+            if (active) m[s] = *reinterpret_cast<const float4*>(a.msg_in + prog.pos_in[t.pos_base + s] * a.ld_m + 4 * q);
         }
     }
     const NoiseQuad nq = noise_quad(a.q0 + static_cast<uint32_t>(q), a.key);
@@ -818,7 +822,8 @@ __device__ __noinline__ void fused_steps_wide(const Program& prog, const ModelAr
     const NoiseQuad nq = noise_quad(a.q0 + static_cast<uint32_t>(q), a.key);
     float4* const first = buf + (parity ? 0 : buf_len) + t.in;
     for (int s = 0; s < t.deg; ++s)
-        first[s * qb] = active ? ld_stream(a.msg_in + prog.pos_in[t.pos_base + s] * a.ld_m + 4 * q) : zero;
+        first[s * qb] =
+            active ? *reinterpret_cast<const float4*>(a.msg_in + prog.pos_in[t.pos_base + s] * a.ld_m + 4 * q) : zero;
     for (int j = 0; j < fs.k; ++j) {
         float4* const cur = buf + (parity ? buf_len : 0);
         const float4* const prev = buf + (parity ? 0 : buf_len) + t.in;

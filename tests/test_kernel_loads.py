@@ -42,3 +42,25 @@ def test_counters_are_not_read_through_the_non_coherent_path():
     for name in ("device.cuh", "step_kernels.cu", "relaysum.cu"):
         for arg in _non_coherent_arguments(_source(name)):
             assert "counts" not in arg, (name, arg)
+
+
+def _body(text: str, name: str) -> str:
+    """The body of the function `name`."""
+    at = re.search(r"\b%s\([^;{]*\)\s*\{" % name, text).end()
+    depth = 1
+    for k in range(at, len(text)):
+        depth += {"{": 1, "}": -1}.get(text[k], 0)
+        if depth == 0:
+            return text[at:k]
+    raise AssertionError("unbalanced braces")
+
+
+def test_multi_step_kernel_reads_what_it_writes_with_ordinary_loads():
+    """relay_steps leaves the messages of its last two steps in both message
+    buffers, the one it starts from included, and updates the models and the
+    optimiser state in place: only the centres stay as they are."""
+    text = _source("step_kernels.cu")
+    args = []
+    for name in ("fused_steps", "fused_steps_wide", "relay_fused_steps_kernel"):
+        args += _non_coherent_arguments(_body(text, name))
+    assert args and all(arg.startswith("a.mu ") for arg in args), args
