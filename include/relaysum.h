@@ -393,8 +393,10 @@ int relay_program(const relay_handle *h, int32_t *nslots, int32_t *order, int32_
  * xbar, mubar are the worker averages (the quantities of Section 4's
  * analysis; mubar is the optimum of f = 1/n sum_i f_i).  out: device double
  * [2]; workspace: device double [relay_metrics_workspace(h)], caller-owned
- * scratch for per-block partial sums, overwritten by every call.  Reduced in
- * double in a fixed order: deterministic.  Needs a bound objective. */
+ * scratch for per-block partial sums, overwritten by every call.  The sums
+ * over the workers are compensated fp32 pairs (about 48 bits), those over the
+ * coordinates double, all in a fixed order: deterministic.  Needs a bound
+ * objective. */
 int64_t relay_metrics_workspace(const relay_handle *h);
 int relay_metrics(relay_handle *h, const float *x, double *workspace, double *out,
                   relay_stream_t stream);

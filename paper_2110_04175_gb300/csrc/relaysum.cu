@@ -143,27 +143,51 @@ struct HiLo {
     Pair hi, lo;
 };
 
-// (s + c) / n: the product with 1 / n as a pair of its own.
+// (s + c) / n: the product with 1 / n as a pair of its own.  s may be smaller
+// than c, where large values cancelled.
 __device__ __forceinline__ HiLo worker_mean(const PairSum& sum, Pair inv_hi, Pair inv_lo) {
     const Pair t = add2(sum.s, sum.c);
-    const Pair e = sub2(sum.c, sub2(t, sum.s));
+    const Pair e = sum_error(sum.s, sum.c, t);
     const Pair p = mul2(t, inv_hi);
     const Pair r = fma2(e, inv_hi, fma2(t, inv_lo, fma2(t, inv_hi, mul2(p, pack(-1.0f)))));
     const Pair hi = add2(p, r);
     return HiLo{hi, sub2(r, sub2(hi, p))};
 }
 
-// Adds the squares (xbar - mubar)^2 of the two coordinates: the difference as
-// an fp32 pair, squared in double.
-__device__ __forceinline__ void add_squared_difference(const HiLo& x, const HiLo& m, double& total) {
-    const Pair minus_m = mul2(m.hi, pack(-1.0f));
-    const Pair t = add2(x.hi, minus_m);
-    const Pair el = add2(sum_error(x.hi, minus_m, t), sub2(x.lo, m.lo));
-    float t0, t1, l0, l1;
-    unpack(t, t0, t1);
-    unpack(el, l0, l1);
-    const double e0 = static_cast<double>(t0) + static_cast<double>(l0);
-    const double e1 = static_cast<double>(t1) + static_cast<double>(l1);
+// Adds (n (xbar - mubar))^2 of the two coordinates, from their sums over the
+// workers.  The sums are subtracted before they are divided, so a mean next to
+// the optimum keeps its bits.  (x.s - m.s) + (x.c - m.c) is h + l exactly
+// wherever the rest l2 is 0, as for values of like magnitude; where it is not
+// (or not finite), the four parts are added in double, at 9 instead of 4
+// double instructions a coordinate (which always taken makes 208 us of
+// metrics for one worker at d = 2.0e7 into 352).
+__device__ __forceinline__ void add_squared_difference(const PairSum& x, const PairSum& m, double& total) {
+    const Pair minus_ms = mul2(m.s, pack(-1.0f)), minus_mc = mul2(m.c, pack(-1.0f));
+    const Pair t = add2(x.s, minus_ms), u = add2(x.c, minus_mc);
+    const Pair te = sum_error(x.s, minus_ms, t), ue = sum_error(x.c, minus_mc, u);
+    const Pair h = add2(t, u);
+    const Pair r = sum_error(t, u, h);
+    const Pair l = add2(r, te);
+    const Pair l2 = add2(sum_error(r, te, l), ue);
+    float h0, h1, l0, l1, r0, r1;
+    unpack(h, h0, h1);
+    unpack(l, l0, l1);
+    unpack(l2, r0, r1);
+    double e0, e1;
+    if (r0 == 0.0f && r1 == 0.0f) {
+        e0 = static_cast<double>(h0) + static_cast<double>(l0);
+        e1 = static_cast<double>(h1) + static_cast<double>(l1);
+    } else {
+        float xs[2], xc[2], ms[2], mc[2];
+        unpack(x.s, xs[0], xs[1]);
+        unpack(x.c, xc[0], xc[1]);
+        unpack(m.s, ms[0], ms[1]);
+        unpack(m.c, mc[0], mc[1]);
+        e0 = (static_cast<double>(xs[0]) - static_cast<double>(ms[0])) +
+             (static_cast<double>(xc[0]) - static_cast<double>(mc[0]));
+        e1 = (static_cast<double>(xs[1]) - static_cast<double>(ms[1])) +
+             (static_cast<double>(xc[1]) - static_cast<double>(mc[1]));
+    }
     total += e0 * e0;
     total += e1 * e1;
 }
@@ -196,10 +220,13 @@ __device__ __forceinline__ float4 within(float4 v, int64_t c, int64_t d) {
     return v;
 }
 
-// Bound by issue and the second read of x (from L2 in part): 1,156 us for 64
+// Bound by issue and the second read of x (from L2 in part): 1,080 us for 64
 // workers at d = 9.2M, 1,523 with scalar arithmetic and the means in double.
-// Keeping a quad's x_i in shared memory between the passes, filled by
-// asynchronous copies, left one block of 4 warps per SM and 1,214 us.
+// The distance to the optimum is added before the second pass, so the sums of
+// the centres hold no registers through it (behind it: 1,196 us).  Keeping a
+// quad's x_i in shared memory between the passes, filled by asynchronous
+// copies, left one block of 4 warps per SM and took 58 us more than reading
+// them again.
 template <int OBJ>
 __global__ void __launch_bounds__(kMetricsThreads, kMetricsResident)
 relay_metrics_kernel(const __grid_constant__ Objective obj, const __grid_constant__ PhiloxKey mu_key,
@@ -221,6 +248,8 @@ relay_metrics_kernel(const __grid_constant__ Objective obj, const __grid_constan
             ms[0].add(pack(mv.x, mv.y));
             ms[1].add(pack(mv.z, mv.w));
         }
+        add_squared_difference(xs[0], ms[0], dist);
+        add_squared_difference(xs[1], ms[1], dist);
         const HiLo xbar[2] = {worker_mean(xs[0], inv_hi, inv_lo), worker_mean(xs[1], inv_hi, inv_lo)};
         const Pair minus_hi[2] = {mul2(xbar[0].hi, pack(-1.0f)), mul2(xbar[1].hi, pack(-1.0f))};
         SquareSum sq[2];
@@ -230,8 +259,6 @@ relay_metrics_kernel(const __grid_constant__ Objective obj, const __grid_constan
             sq[1].add(pack(xv.z, xv.w), minus_hi[1], xbar[1].lo);
         }
         add_quad(HiLo{sq[0].sq.s, add2(sq[0].sq.c, sq[0].lo)}, HiLo{sq[1].sq.s, add2(sq[1].sq.c, sq[1].lo)}, xi);
-        add_squared_difference(xbar[0], worker_mean(ms[0], inv_hi, inv_lo), dist);
-        add_squared_difference(xbar[1], worker_mean(ms[1], inv_hi, inv_lo), dist);
     }
     const double bxi = block_sum(xi, red);
     const double bdist = block_sum(dist, red);
@@ -331,7 +358,8 @@ int launch_metrics(const relay_handle* h, const ModelArgs& a, int max_blocks, do
     if (rc != RELAY_OK) return rc;
     const double denom = h->d > 0 ? static_cast<double>(h->d) : 1.0;
     return launch_step_kernel(relay_metrics_finish_kernel, 1, kMetricsThreads, 0, stream, true,
-                              static_cast<const double*>(workspace), blocks, 1.0 / (n * denom), 1.0 / denom, out);
+                              static_cast<const double*>(workspace), blocks, 1.0 / (n * denom),
+                              1.0 / (static_cast<double>(n) * n * denom), out);  // dist carries n^2
 }
 
 // Rows of a message buffer: E, plus one received-sum row per wide node when

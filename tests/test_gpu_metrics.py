@@ -1,5 +1,7 @@
 """Convergence metrics (relay_metrics): the consensus distance and the
 distance of the average model to the optimum, as in the paper's analysis."""
+from fractions import Fraction
+
 import numpy as np
 import pytest
 import torch
@@ -99,3 +101,78 @@ def test_metrics_at_the_edges_of_their_blocks(n, d):
     for _ in range(2):
         regenerated.step(0.2, 4)
     assert np.array_equal(regenerated.metrics()[0].cpu().numpy(), m)
+
+
+def _exact_distance(x, mu):
+    """mean_c (xbar - mubar)^2 of float32 arrays in rational arithmetic."""
+    diff = [sum(map(Fraction, map(float, x[:, c]))) - sum(map(Fraction, map(float, mu[:, c])))
+            for c in range(x.shape[1])]
+    return sum(v * v for v in diff) / (x.shape[0] ** 2 * x.shape[1])
+
+
+def _metrics_of(x, mu):
+    n, d = x.shape
+    run = rs.RelayRun(n, d, wl.random_tree(n, 2), device="cuda:0")
+    run.init(0.0, 4, wl.identity_mix(n), 0.0, 5, 0.0)
+    run.x[:, :d] = torch.from_numpy(x)
+    run.mu[:, :d] = torch.from_numpy(mu)
+    return run.metrics()[0].cpu().numpy()
+
+
+@pytest.mark.parametrize("n", [1, 3, 7, 24, 64])
+@pytest.mark.parametrize("d", [5, 2051])
+@pytest.mark.parametrize("gap", [1.0, 1e-4])
+def test_distance_next_to_the_optimum(n, d, gap):
+    """The average model close to the optimum, where a converging run ends.
+    All values lie on a grid of 2^-20 below 8 and n <= 64, so the sums over
+    the workers have at most 29 bits and their fp32 pairs are exact.  What
+    remains is the rounding of the squares, of their sums (4 in a thread, 13
+    over a block, 13 over the blocks) and of the scaling: under 40 roundings
+    of 2^-53, all of positive terms."""
+    rng = np.random.Generator(np.random.PCG64(n + d))
+    grid = 2.0 ** -20
+    mu = np.clip(rng.standard_normal((n, d)), -4, 4)
+    x = mu.mean(axis=0) + gap * rng.standard_normal(d) + 1e-2 * rng.standard_normal((n, d))
+    x, mu = (np.round(np.clip(v, -7.9, 7.9) / grid).astype(np.float64) * grid for v in (x, mu))
+    x, mu = x.astype(np.float32), mu.astype(np.float32)
+    want = _exact_distance(x, mu)
+    got = Fraction(float(_metrics_of(x, mu)[1]))
+    assert abs(got - want) <= 40 * Fraction(2) ** -53 * want, float((got - want) / want)
+
+
+def test_distance_where_large_values_cancel():
+    """A column's running sum (1e-3) ends below the rounding error that it
+    gathered on the way (1.3): both are exact here, so the bar is the one
+    above."""
+    x = np.array([[1e8, 3e7, -2e8], [1.3, 0.7, 5.3], [-1e8, -3e7, 2e8], [1e-3, 2e-3, 3e-3]], np.float32)
+    mu = np.zeros_like(x)
+    want = _exact_distance(x, mu)
+    got = Fraction(float(_metrics_of(x, mu)[1]))
+    assert abs(got - want) <= 40 * Fraction(2) ** -53 * want, float((got - want) / want)
+
+
+def test_distance_over_many_orders_of_magnitude():
+    """Workers whose values differ by up to 2^40, so that a difference does
+    not fit two fp32 values.  A worker sum gathers at most n rounding errors,
+    each within 2^-24 of the largest partial sum, and rounds every addition of
+    them: n^2 2^-48 sum_i |x_i| for its pair.  Behind that, the roundings of
+    test_distance_next_to_the_optimum."""
+    n, d = 6, 2051
+    rng = np.random.Generator(np.random.PCG64(9))
+    scale = np.exp2(-rng.integers(0, 41, size=(n, d)).astype(np.float64))
+    x = (rng.standard_normal((n, d)) * scale).astype(np.float32)
+    mu = (rng.standard_normal((n, d)) * scale[::-1]).astype(np.float32)
+    want = _exact_distance(x, mu)
+    diff = np.abs(x.astype(np.float64).sum(axis=0) - mu.astype(np.float64).sum(axis=0))
+    delta = n ** 2 * 2.0 ** -48 * (np.abs(x).sum(axis=0, dtype=np.float64) + np.abs(mu).sum(axis=0, dtype=np.float64))
+    bound = float(np.sum(2 * diff * delta + delta ** 2)) / (n * n * d) + 40 * 2.0 ** -53 * float(want)
+    got = Fraction(float(_metrics_of(x, mu)[1]))
+    assert abs(float(got - want)) <= bound, (float((got - want) / want), bound / float(want))
+
+
+def test_distance_beyond_fp32_range():
+    x = np.array([[3e38, 1.0, -3e38, 2e38]], np.float32)
+    mu = np.array([[-3e38, 1.5, 3e38, 2e38]], np.float32)
+    want = _exact_distance(x, mu)
+    got = Fraction(float(_metrics_of(x, mu)[1]))
+    assert abs(got - want) <= 40 * Fraction(2) ** -53 * want, float((got - want) / want)
