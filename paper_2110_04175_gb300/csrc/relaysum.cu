@@ -203,6 +203,15 @@ __device__ __forceinline__ void add_quad(const HiLo& a, const HiLo& b, double& t
     unpack(t, t0, t1);
     unpack(e, e0, e1);
     const float s = __fadd_rn(t0, t1);
+    if (!isfinite(s)) {  // beyond fp32's range together: one by one
+        float v[4], w[4];
+        unpack(a.hi, v[0], v[1]);
+        unpack(b.hi, v[2], v[3]);
+        unpack(a.lo, w[0], w[1]);
+        unpack(b.lo, w[2], w[3]);
+        for (int k = 0; k < 4; ++k) total += static_cast<double>(v[k]) + static_cast<double>(w[k]);
+        return;
+    }
     const float bb = __fsub_rn(s, t0);
     const float err = __fadd_rn(__fsub_rn(t0, __fsub_rn(s, bb)), __fsub_rn(t1, bb));
     total += static_cast<double>(s);

@@ -176,3 +176,12 @@ def test_distance_beyond_fp32_range():
     want = _exact_distance(x, mu)
     got = Fraction(float(_metrics_of(x, mu)[1]))
     assert abs(got - want) <= 40 * Fraction(2) ** -53 * want, float((got - want) / want)
+
+
+def test_consensus_distance_of_a_quad_beyond_fp32_range():
+    """Each coordinate's squares sum to 2e38, the four of a quad to 8e38.  The
+    pair arithmetic is within 2^-40 for the two workers."""
+    x = np.array([[1e19, -1e19, 1e19, 1e19], [-1e19, 1e19, -1e19, -1e19]], np.float32)
+    got = _metrics_of(x, np.zeros_like(x))
+    want = float(np.float32(1e19)) ** 2
+    assert abs(got[0] - want) <= 2.0 ** -40 * want and got[1] == 0.0, got
