@@ -519,7 +519,10 @@ __device__ __forceinline__ NodeThread node_thread(const Program& prog, const Mod
 }
 
 // Outgoing message s = prefix(s) + suffix(s + 1) with prefix(s) = xh + m_0 +
-// ... + m_{s-1}; the zeros of a lane's missing neighbours add nothing.
+// ... + m_{s-1}.  A lane's missing neighbours hold nothing4(): v + -0 is v for any
+// v, a zero's sign included (-0 + 0 would be +0).
+__device__ __forceinline__ float4 nothing4() { return make_float4(-0.0f, -0.0f, -0.0f, -0.0f); }
+
 template <int D>
 __device__ __forceinline__ void narrow_messages(const float4 (&m)[D], float4 xh, uint32_t lost_bits,
                                                 float4 (&o)[D]) {
@@ -552,7 +555,7 @@ __device__ __forceinline__ float4 node_send(const Program& prog, const ModelArgs
     auto request = [&]() {
 #pragma unroll
         for (int s = 0; s < D; ++s) {
-            m[s] = make_float4(0.f, 0.f, 0.f, 0.f);
+            m[s] = nothing4();
             if (s < t.deg) m[s] = ld_stream(a.msg_in + prog.pos_in[t.pos_base + s] * a.ld_m + 4 * q);
         }
     };
@@ -750,12 +753,11 @@ __device__ __forceinline__ void fused_steps(const Program& prog, const ModelArgs
                                             int qb, int& parity, bool active, int64_t q, float4& xv, float4 mv,
                                             float4& m1, float4& m2) {
     constexpr int DN = D > 0 ? D : 1;
-    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
     float4 m[DN];
     int out[DN];
 #pragma unroll
     for (int s = 0; s < D; ++s) {
-        m[s] = zero;
+        m[s] = nothing4();
         out[s] = 0;
         if (s < t.deg) {
             // where the message to neighbour s arrives

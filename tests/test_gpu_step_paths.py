@@ -83,3 +83,31 @@ def test_steps_from_any_counters(shape, n, k, algorithm):
     _same(*runs)
     if algorithm == "dme":
         assert torch.equal(runs[0].trees[0].dme_count, runs[1].trees[0].dme_count)
+
+
+# 24 and 40 workers: warps whose workers differ in degree
+@pytest.mark.parametrize("n", [2, 5, 24, 40])
+def test_paths_agree_in_the_sign_of_zero(n):
+    """Models, messages and centres at -0 and 0 without noise: the sums are
+    zeros of either sign, and a lane with fewer neighbours than its warp's
+    widest must add nothing for the missing ones."""
+    d, edges = 77, wl.random_tree(n, 3)
+    runs = {}
+    for kernel in ("walk", "nodes", "steps"):
+        run = rs.RelayRun(n, d, edges, device="cuda:0", mode=1, kernel="walk" if kernel == "walk" else "nodes",
+                          received_sums=False)
+        run.init(0.0, 3, wl.identity_mix(n), 0.0, 5, 0.0)
+        run.mu.zero_()
+        for t in (run.x, run.msg[0], run.msg[1]):
+            t.fill_(-0.0)
+        if kernel == "steps":
+            run.steps(3, 0.05, 3)
+        else:
+            for _ in range(3):
+                run.step(0.05, 3)
+        runs[kernel] = run
+    walk = runs["walk"]
+    assert bool((walk.x[:, :d].view(torch.int32) != 0).any()) and not bool(walk.x[:, :d].any())
+    for other in (runs["nodes"], runs["steps"]):
+        for a, b in ((walk.x, other.x), (walk.messages[:walk.E], other.messages[:walk.E])):
+            assert torch.equal(a[:, :d].view(torch.int32), b[:, :d].view(torch.int32))
