@@ -62,11 +62,12 @@ def test_initial_model_and_centres_match_oracle_normals():
 
 
 def test_normal_generator_error_within_derived_bound():
-    """The GPU's normals against the oracle's fp64 Box-Muller of the same
-    Philox uniforms, on 8.4M draws (the centres of 8 workers over 2^20
+    """The GPU's normals of the centres against the oracle's fp64 Box-Muller of
+    the same Philox uniforms, on 8.4M draws (the centres of 8 workers over 2^20
     coordinates, mu_i = N_i with an identity mixture): every one within
     gpu_util.NORMAL_ABS_ERR, the bound derived from the GPU's logf,
-    sqrt.approx and __sincosf.  The error is small on average too."""
+    sqrt.approx and __sincosf.  The error is small on average too.  The
+    gradient noise has its own path: the next test."""
     n, d = 8, 1 << 20
     run = rs.RelayRun(n, d, wl.chain(n), device="cuda:0")
     run.init(0.0, 0, wl.identity_mix(n), 1.0, 12345, 0.0)
@@ -77,6 +78,37 @@ def test_normal_generator_error_within_derived_bound():
     assert err.max() <= NORMAL_ABS_ERR, err.max()
     assert err.mean() <= 0.1 * NORMAL_ABS_ERR, err.mean()
     assert np.abs(want).max() > 5.0  # the draws reach the tails, where r is largest
+
+
+@pytest.mark.parametrize("kernel", ["walk", "nodes", "steps"])
+def test_noise_generator_error_within_derived_bound(kernel):
+    """The same for the gradient noise (stream 0: the logarithm by polynomial,
+    the split Philox rounds), every worker's normals at a step past the first.
+    With every message lost and x = mu = 0, sigma = lr = 1, one step leaves
+    x_i = -xi_i exactly.  8.4M draws reach u below 2^-22 and above 1 - 2^-22,
+    and their error is no larger than that of the centres' normals, which use
+    CUDA's logf."""
+    n, d, t = 8, 1 << 20, 5
+    run = rs.RelayRun(n, d, wl.chain(n), device="cuda:0", mode=0, kernel="walk" if kernel == "walk" else "nodes")
+    run.init(0.0, 12345, wl.identity_mix(n), 1.0, 12345, 1.0)
+    centres = run.mu[:, :d].double().cpu().numpy()
+    run.mu.zero_()
+    run.set_lost(np.ones(2 * (n - 1), np.uint8))
+    run.t = t
+    if kernel == "steps":
+        run.steps(1, 1.0, 12345)
+    else:
+        run.step(1.0, 12345)
+    torch.cuda.synchronize()
+    got = -run.x[:, :d].double().cpu().numpy()
+    want = np.stack(parallel_map(lambda i: oracle.normals(12345, 0, d, row=i, step=t, stream=0), range(n)))
+    err = np.abs(got - want)
+    assert err.max() <= NORMAL_ABS_ERR, err.max()
+    assert err.mean() <= 0.1 * NORMAL_ABS_ERR, err.mean()
+    assert np.abs(want).max() > 5.0
+    want = np.stack(parallel_map(lambda i: oracle.normals(12345, 0, d, row=i, step=0, stream=1), range(n)))
+    rms, rms_centres = (float(np.sqrt(np.mean(e ** 2))) for e in (err, centres - want))
+    assert rms <= 1.01 * rms_centres, (rms, rms_centres)  # 1%: far above the spread of 8.4M squares
 
 
 def test_gradient_noise_stream():
