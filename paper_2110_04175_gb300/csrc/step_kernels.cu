@@ -462,7 +462,7 @@ __device__ __forceinline__ void walk(const Program& prog, const ModelArgs& a, co
 // budgeted for (0: no bound, the compiler's choice: 64 registers, 8 CTAs).
 // The wide-node variant takes 8: 5.90 ms per step on the 64-worker star at d =
 // 2.5e7, against 6.14 ms budgeted for 7, 6.57 for 6 and 7.38 for 9 (which
-// spills).  Narrow trees with stored centres take 0 or 7 (walk_budget).
+// spills).  Narrow trees with stored centres take 0 or 7 (seven_ctas).
 template <int OBJ, int OPT, int NT, bool WIDE, int MIN>
 __global__ void __launch_bounds__(128, MIN)
 relay_models_kernel(const __grid_constant__ Windows<NT> win, const __grid_constant__ ObjectiveArg<OBJ> obj,
@@ -994,19 +994,31 @@ int models_threads(int nslots) {
     return t;
 }
 
+// Threads per CTA and shared memory of the walk over NT handles' windows,
+// sized for the larger program.
+struct WalkShape {
+    int threads;
+    size_t smem;
+};
+
+template <int OBJ, int NT>
+WalkShape walk_shape(const relay_handle* const* hs) {
+    int per_thread = 0;
+    for (int k = 0; k < NT; ++k)
+        per_thread = std::max(per_thread, hs[k]->prog.nslots + (OBJ == relaysum::kMuCachedCentres ? hs[k]->obj.K : 0));
+    const int threads = models_threads(per_thread);
+    return WalkShape{threads, static_cast<size_t>(per_thread) * threads * 16};
+}
+
 // The walk over NT handles' windows in one launch (NT = 1: one handle).  The
 // handles share the objective source and the local optimiser (the caller
-// checks); threads and shared memory are sized for the larger program.
+// checks).
 template <int OBJ, int OPT, int NT, bool WIDE, int MIN>
 int launch_models(const relay_handle* const* hs, const ModelArgs* as, cudaStream_t stream, bool after_counts) {
     int dev = 0;
     const int sms = device_sms(&dev);
     if (sms <= 0) return RELAY_ECUDA;
-    int per_thread = 0;
-    for (int k = 0; k < NT; ++k)
-        per_thread = std::max(per_thread, hs[k]->prog.nslots + (OBJ == relaysum::kMuCachedCentres ? hs[k]->obj.K : 0));
-    const int threads = models_threads(per_thread);
-    const size_t smem = static_cast<size_t>(per_thread) * threads * 16;
+    const auto [threads, smem] = walk_shape<OBJ, NT>(hs);
     if (smem > static_cast<size_t>(kMaxSmem)) return RELAY_EUNSUPPORTED;
     if (resident_ctas<relay_models_kernel<OBJ, OPT, NT, WIDE, MIN>>(dev, threads, smem) <= 0) return RELAY_ECUDA;
     Windows<NT> win;
@@ -1051,29 +1063,40 @@ int launch_nodes(const relay_handle* h, const ModelArgs& a, cudaStream_t stream,
                               program_of(h), objective_of<OBJ>(h), mu_key, a, qb_log2);
 }
 
-// Whether the walk over narrow trees with stored centres runs 7 CTAs per SM
-// rather than 8.  Eight are faster over many waves (1107 against 1125 us on
-// the 32-worker binary tree at d = 9.2M), but a short grid's last wave leaves
-// SMs idle, and it is fuller when 7 at a time divide the grid better: the
-// 64-worker torus tree at d = 1.0M is 1.61 waves of 8 or 1.84 of 7 CTAs per SM
-// and takes 283 or 272 us.
-bool seven_ctas(const ModelArgs* as, int windows) {
+// Whether the walk over narrow trees with stored centres takes the build
+// budgeted for 7 CTAs per SM rather than the unbounded one (8 of 128 threads,
+// unless the slots allow fewer).  More CTAs are faster over many waves, but a
+// short grid's last wave leaves SMs idle, and it is fuller when 7 at a time
+// divide the grid better.  Each side at 16 to 64 workers, 7 against 8:
+//   1.6 to 4.0 waves of 8, SGD       0.94 to 1.00 of the time (torus tree of 64
+//                                    workers at d = 1.0M: 272 against 286 us)
+//   the same, Adam                   0.97 to 1.01 (453 against 459 us)
+//   the same, Nesterov               0.98 to 1.025: not worth a build
+//   one wave of 8 or more than four  1.01 to 1.4 (32-worker binary tree at d =
+//                                    9.2M: 1,124 against 1,109 us with SGD)
+template <int OPT, int NT>
+bool seven_ctas(const relay_handle* const* hs, const ModelArgs* as) {
     int dev = 0;
     const int64_t sms = device_sms(&dev);
-    if (sms <= 0) return false;  // the launch reports it
+    const auto [threads, smem] = walk_shape<relaysum::kMuStored, NT>(hs);
+    if (sms <= 0 || smem > static_cast<size_t>(kMaxSmem)) return false;  // the launch reports it
+    const int most = resident_ctas<relay_models_kernel<relaysum::kMuStored, OPT, NT, false, 0>>(dev, threads, smem);
+    const int fewer = resident_ctas<relay_models_kernel<relaysum::kMuStored, OPT, NT, false, 7>>(dev, threads, smem);
+    if (fewer <= 0 || fewer >= most) return false;
     int64_t ctas = 0;
-    for (int k = 0; k < windows; ++k) ctas += (as[k].nquads + 127) / 128;
-    auto rounds = [&](int64_t per_sm) { return (ctas + sms * per_sm - 1) / (sms * per_sm); };
-    // share of the CTA slots that the rounds fill: ctas / (rounds x slots), 7 against 8
-    return 10 * rounds(8) * 8 > 11 * rounds(7) * 7;
+    for (int k = 0; k < NT; ++k) ctas += (as[k].nquads + threads - 1) / threads;
+    auto slots = [&](int64_t per_sm) { return (ctas + sms * per_sm - 1) / (sms * per_sm) * per_sm; };
+    // share of the CTA slots that the waves fill, ctas / (waves x slots): 10 % fuller
+    return 10 * slots(most) > 11 * slots(fewer);
 }
 
 template <int OPT, int NT, bool WIDE>
 int launch_walk_src(const relay_handle* const* hs, const ModelArgs* as, cudaStream_t stream, bool after_counts) {
     switch (hs[0]->obj.source) {
         case relaysum::kMuStored:
-            if (!WIDE && seven_ctas(as, NT))
-                return launch_models<relaysum::kMuStored, OPT, NT, WIDE, WIDE ? 8 : 7>(hs, as, stream, after_counts);
+            if constexpr (!WIDE && OPT != 1)
+                if (seven_ctas<OPT, NT>(hs, as))
+                    return launch_models<relaysum::kMuStored, OPT, NT, WIDE, 7>(hs, as, stream, after_counts);
             return launch_models<relaysum::kMuStored, OPT, NT, WIDE, WIDE ? 8 : 0>(hs, as, stream, after_counts);
         case relaysum::kMuPerRow:
             return launch_models<relaysum::kMuPerRow, OPT, NT, WIDE, WIDE ? 8 : 0>(hs, as, stream, after_counts);
