@@ -1071,7 +1071,8 @@ int launch_nodes(const relay_handle* h, const ModelArgs& a, cudaStream_t stream,
 //   1.6 to 4.0 waves of 8, SGD       0.94 to 1.00 of the time (torus tree of 64
 //                                    workers at d = 1.0M: 272 against 286 us)
 //   the same, Adam                   0.97 to 1.01 (453 against 459 us)
-//   the same, Nesterov               0.98 to 1.025: not worth a build
+//   the same, Nesterov               0.98 to 1.025 (32 workers at d = 1.0M: 182
+//                                    against 185 us; 64 at 1.5M: 554 against 543)
 //   one wave of 8 or more than four  1.01 to 1.4 (32-worker binary tree at d =
 //                                    9.2M: 1,124 against 1,109 us with SGD)
 template <int OPT, int NT>
@@ -1094,7 +1095,7 @@ template <int OPT, int NT, bool WIDE>
 int launch_walk_src(const relay_handle* const* hs, const ModelArgs* as, cudaStream_t stream, bool after_counts) {
     switch (hs[0]->obj.source) {
         case relaysum::kMuStored:
-            if constexpr (!WIDE && OPT != 1)
+            if constexpr (!WIDE)
                 if (seven_ctas<OPT, NT>(hs, as))
                     return launch_models<relaysum::kMuStored, OPT, NT, WIDE, 7>(hs, as, stream, after_counts);
             return launch_models<relaysum::kMuStored, OPT, NT, WIDE, WIDE ? 8 : 0>(hs, as, stream, after_counts);
