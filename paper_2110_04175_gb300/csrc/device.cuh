@@ -326,6 +326,18 @@ __device__ __forceinline__ void allow_dependent_launch() {
 }
 __device__ __forceinline__ void wait_for_prior_grid() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// A counter, behind wait_for_prior_grid(): the counter kernel may write it while
+// this kernel already runs, so not by a non-coherent load, which is defined
+// only for memory that stays as it is for the kernel's lifetime and may be
+// moved ahead of the wait.  Being volatile, it stays behind it.  (A plain load
+// of the array costs the walk over two windows with Adam 68 instead of 64
+// registers, hence a CTA per SM.)
+__device__ __forceinline__ int32_t ld_counter(const int32_t* p) {
+    int32_t v;
+    asm volatile("ld.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+
 // mu_i for quad q: read, or regenerated exactly as relay_fill_mu_kernel
 // writes it (same normals, same fma order), so both sources give the same bits.
 template <int OBJ, typename Obj>

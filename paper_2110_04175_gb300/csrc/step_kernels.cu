@@ -314,17 +314,14 @@ __device__ __forceinline__ void worker_factors(const ModelArgs& a, int n, int nb
     }
 }
 
-// After wait_for_prior_grid(), with ordinary loads: relay_step's counter kernel
-// may still write the counters while this kernel already runs, and a
-// non-coherent load, defined only for memory that stays as it is for the
-// kernel's lifetime, could be moved ahead of the wait.
+// To be called after wait_for_prior_grid().
 __device__ __forceinline__ void rebuild_factors(const Program& prog, const ModelArgs& a, float* s_scale,
                                                 float* s_fill) {
     const int n = prog.n;
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
         const NodeRec r = prog.node[i];
         int nbar = 1;
-        for (int p = 0; p < r.deg; ++p) nbar += a.counts[prog.pos_in[r.pos_base + p]];
+        for (int p = 0; p < r.deg; ++p) nbar += ld_counter(a.counts + prog.pos_in[r.pos_base + p]);
         worker_factors(a, n, nbar, s_scale[i], s_fill[i]);
     }
 }
