@@ -37,3 +37,14 @@ struct relay_handle {
     bool rsum = false;
     uint32_t lost[relaysum::kMaxE / 32 + 1] = {};
 };
+
+namespace relaysum {
+
+// Whether the handle's tree has a node of degree > kRegDeg (a wide node).
+inline bool has_wide(const relay_handle* h) {
+    for (int i = 0; i < h->prog.n; ++i)
+        if (h->prog.node[i].deg > kRegDeg) return true;
+    return false;
+}
+
+}  // namespace relaysum

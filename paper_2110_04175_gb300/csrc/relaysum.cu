@@ -23,9 +23,9 @@
 #include <cstring>
 #include <new>
 
+using relaysum::has_wide;
 using relaysum::kMaxE;
 using relaysum::kMaxN;
-using relaysum::kRegDeg;
 using relaysum::NodeRec;
 using relaysum::Objective;
 using relaysum::Program;
@@ -319,16 +319,7 @@ bool use_nodes(const relay_handle* h) {
     if (h->kernel == RELAY_KERNEL_NODES) return true;
     if (h->kernel == RELAY_KERNEL_WALK) return false;
     if (h->nquads * h->prog.n >= kNodesBelowWorkerQuads) return false;
-    for (int i = 0; i < h->prog.n; ++i)
-        if (h->prog.node[i].deg > kRegDeg) return false;
-    return true;
-}
-
-// Whether a tree has a node of degree > kRegDeg (the walk's WIDE variant).
-bool has_wide(const relay_handle* h) {
-    for (int i = 0; i < h->prog.n; ++i)
-        if (h->prog.node[i].deg > kRegDeg) return true;
-    return false;
+    return !has_wide(h);
 }
 
 // relay_steps takes the multi-step kernel unless the walk is forced or, under
@@ -342,9 +333,7 @@ bool use_fused(const relay_handle* h) {
     if (h->prog.nwide > 0) return false;  // received-sum rows are kept by the per-step kernels only
     if (h->kernel == RELAY_KERNEL_NODES) return true;
     if (h->kernel == RELAY_KERNEL_WALK) return false;
-    for (int i = 0; i < h->prog.n; ++i)
-        if (h->prog.node[i].deg > kRegDeg) return false;
-    return true;
+    return !has_wide(h);
 }
 
 // Whether the launches for few workers (smaller parameters) take this handle.

@@ -30,6 +30,7 @@
 #include <cstring>
 #include <type_traits>
 
+using relaysum::has_wide;
 using relaysum::kRegDeg;
 using relaysum::NodeRec;
 
@@ -974,13 +975,6 @@ const Program& program_of(const relay_handle* h) { return pick(h, static_cast<co
 template <int OBJ>
 ObjectiveArg<OBJ> objective_of(const relay_handle* h) {
     return pick(h, static_cast<const ObjectiveArg<OBJ>*>(nullptr));
-}
-
-// Whether a tree has a node of degree > kRegDeg (the walk's WIDE variant).
-bool has_wide(const relay_handle* h) {
-    for (int i = 0; i < h->prog.n; ++i)
-        if (h->prog.node[i].deg > kRegDeg) return true;
-    return false;
 }
 
 // Threads per CTA for the fused kernel: 128, fewer when the slots would not
