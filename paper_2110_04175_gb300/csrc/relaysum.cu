@@ -306,15 +306,17 @@ bool overlap(const void* a, int64_t abytes, const void* b, int64_t bbytes) {
 
 // AUTO picks the node-parallel kernel below this many worker-quads (n times
 // the quads) when no worker has more than kRegDeg neighbours.  Measured on
-// one GB300 (whole step, L2 flushed, n = 8 to 64): the node kernel is ahead
-// below about 2^21 worker-quads on chains, binary trees and the torus tree
-// and even or behind above; on a star one thread carries the hub's edges
-// while its CTA waits, so the walk stays faster there.
+// one GB300 (whole step, L2 flushed), the node kernel against the walk: ahead
+// up to 2^16.1 to 2^16.5 quads, 2^19.5 worker-quads with 8 workers and 2^22 with
+// 64.  The line meets that at 24 to 32 workers (binary tree of 32 at 2^21: 48
+// against 54 us).  With 8 it is late (at 2^20: 27.4 against 25.7 us), with 64
+// early (chain at 2^21: 52 against 88 us).  On a star one thread carries the
+// hub's edges while its CTA waits, so the walk is faster there.
 constexpr int64_t kNodesBelowWorkerQuads = int64_t(1) << 21;
 
 // AUTO: the walk keeps every array's traffic at one pass with one thread
-// per quad; below about one resident wave of those threads the GPU idles,
-// and the node-parallel form (n threads per quad) is used instead.
+// per quad; with much less than a resident wave of those threads the GPU
+// idles, and the node-parallel form (n threads per quad) is used instead.
 bool use_nodes(const relay_handle* h) {
     if (h->kernel == RELAY_KERNEL_NODES) return true;
     if (h->kernel == RELAY_KERNEL_WALK) return false;
@@ -327,8 +329,8 @@ bool use_nodes(const relay_handle* h) {
 // all its edges at every step while the rest of the CTA waits at the
 // barrier (a 64-worker star measured 3.7x slower than one relay_step per
 // step).  Measured on one GB300 with every degree <= kRegDeg, from 8 workers
-// and d = 4096 to 32 workers and d = 1.1e8, the multi-step kernel was ahead
-// everywhere (1.2x to 1.8x).
+// and d = 4096 to 32 workers and d = 1.1e8, 64 steps per call, the multi-step
+// kernel is ahead everywhere: 2.2x to 2.8x, 9x for the 8 workers at d = 4096.
 bool use_fused(const relay_handle* h) {
     if (h->prog.nwide > 0) return false;  // received-sum rows are kept by the per-step kernels only
     if (h->kernel == RELAY_KERNEL_NODES) return true;

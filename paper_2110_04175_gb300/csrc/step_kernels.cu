@@ -365,11 +365,12 @@ struct Windows {
 // them drift apart, which cost HBM locality and left a last partial round
 // (13.35 -> 12.86 ms per step on the 32-worker binary tree at d = 1.1e8, 580
 // -> 539 us on two 16-worker trees at d = 9.2M, 787 -> 683 us on the 16-worker
-// chain with regenerated centres).  OBJ: where mu
-// comes from (ObjectiveSource).  OPT: the local optimiser (0 SGD, 1 Nesterov
-// momentum, 2 Adam).  WIDE: some node has more than kRegDeg neighbours;
-// without one the wide-node paths are not compiled, and they cost the narrow
-// trees nothing.
+// chain with regenerated centres).  A grid just past a whole number of waves
+// loses a little to it (24-worker chain at d = 1.25M, 2.02 waves: 140.5 -> 142.5
+// us).  OBJ: where mu comes from (ObjectiveSource).  OPT: the local optimiser
+// (0 SGD, 1 Nesterov momentum, 2 Adam).  WIDE: some node has more than kRegDeg
+// neighbours; without one the wide-node paths are not compiled, and they cost
+// the narrow trees nothing.
 template <int OBJ, int OPT, bool WIDE>
 __device__ __forceinline__ void walk(const Program& prog, const ModelArgs& a, const ObjectiveArg<OBJ>& obj,
                                      const PhiloxKey& mu_key, int64_t cta, float4* slot_mem, float* s_scale,
@@ -544,7 +545,9 @@ __device__ __forceinline__ void narrow_messages(const float4 (&m)[D], float4 xh,
 // Phase 1 of a worker with at most D <= kRegDeg neighbours: its incoming rows
 // are requested before the noise arithmetic, which covers their latency (with
 // Adam after its update, whose registers they would spill: 40.7 against 40.2
-// us on the 16-worker chain at d = 272,474).  `sent[s]` is the float4 index where the message to neighbour s arrives.
+// us on the 16-worker chain at d = 272,474).  `sent[s]` is the float4 index
+// where the message to neighbour s arrives; Adam looks it up again instead of
+// holding it (8 bytes spilled, 36 otherwise).
 template <int D, int OPT>
 __device__ __forceinline__ float4 node_send(const Program& prog, const ModelArgs& a, const NodeThread& t, int64_t q,
                                             float4 xv, float4 mv, const int (&sent)[kRegDeg], int qb, float4* m_new) {
@@ -881,12 +884,14 @@ __device__ __noinline__ void fused_steps_wide(const Program& prog, const ModelAr
 // CTA advances them once, before its first quads.
 //
 // THREADS: up to 32 workers take CTAs of at most 256 threads, three per SM
-// with 80 registers, where the barrier holds fewer warps and nothing spills
-// in the loop: against 512 threads, two per SM with 64 registers, 510 -> 491
-// us (16-worker binary tree, d = 272,474, 64 steps), 30.7 -> 28.7 us (8-worker
-// chain, d = 4,096), 806 -> 785 us with Adam.  More workers keep 512, since
-// half of it would leave rows of 4 quads: 362 against 351 us on the 64-worker
-// chain at d = 30,001.
+// with 80 registers, where the barrier holds fewer warps and less spills
+// (nothing with SGD, 4 bytes with Nesterov and 36 with Adam, against 84 to 176
+// with 64 registers): against 512 threads, two per SM with 64 registers, 510 ->
+// 491 us (16-worker binary tree, d = 272,474, 64 steps), 30.7 -> 28.7 us
+// (8-worker chain, d = 4,096), 806 -> 785 us with Adam.  More workers keep 512,
+// since half of it would leave rows of 4 quads: 362 against 351 us on the
+// 64-worker chain at d = 30,001.  Every build has a stack frame, for the
+// arguments that fused_steps_wide takes by reference.
 constexpr int kFusedFewWorkers = 32;
 constexpr int fused_threads(int n) { return n <= kFusedFewWorkers ? 256 : 512; }
 
@@ -1064,7 +1069,8 @@ int launch_nodes(const relay_handle* h, const ModelArgs& a, cudaStream_t stream,
 //   the same, Adam                   0.97 to 1.01 (453 against 459 us)
 //   the same, Nesterov               0.98 to 1.025 (32 workers at d = 1.0M: 182
 //                                    against 185 us; 64 at 1.5M: 554 against 543)
-//   one wave of 8 or more than four  1.01 to 1.4 (32-worker binary tree at d =
+//   0.9 to 1 wave of 8               1.2 to 1.4
+//   more than four                   1.01 to 1.06 (32-worker binary tree at d =
 //                                    9.2M: 1,124 against 1,109 us with SGD)
 template <int OPT, int NT>
 bool seven_ctas(const relay_handle* const* hs, const ModelArgs* as) {
